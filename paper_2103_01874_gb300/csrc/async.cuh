@@ -21,6 +21,13 @@ __device__ __forceinline__ void cp_async(void* smem, const void* gmem) {
   if (BYTES == 16) cp_async16(smem, gmem);
   else cp_async8(smem, gmem);
 }
+// groups: the copies issued since the last commit form one; wait_group<N> waits
+// for all but the thread's N newest
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait_group() {
+  asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
+}
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
 }  // namespace ppe

@@ -18,12 +18,13 @@
 //
 // Representation: value = hi + lo, |lo| <= ulp(hi)/2 after normalisation.
 // Relative precision ~2^-48 (3.6e-15).  Range: magnitudes in [2^-74, 2^127];
-// smaller inputs are flushed to zero (their contribution is below 1e-22 in
-// absolute value), larger ones are out of scope.
+// below that the low part thins out (denormal) and magnitudes under 2^-126
+// are flushed to a few 1e-45, larger ones are out of scope.
 //
 // d2df(x): hi = x truncated to 24 significant bits (exponent rebias and
 // mantissa shift on the bit pattern), lo = the remaining 29 mantissa bits as an
-// integer, converted with one int->float conversion and scaled by 2^(e-1075).
+// integer, converted with one int->float conversion and scaled by two factors,
+// 2^-52 and the power of two of hi.
 // df2d(a): the exact doubles of hi and lo from their bit patterns, added by
 // one FP64 add (correctly rounded; four per cell in the correction, well
 // within the FP64 pipe those kernels otherwise leave idle).  df2d_alu(a), for
@@ -112,9 +113,18 @@ PPE_HD df fast_two_sum(float a, float b) {
   const float e = b - (s - a);
   return {s, e};
 }
+// a b rounded once, never contracted into a following sum: the exact forms
+// below subtract the rounded product again
+PPE_HD float mul_rn(float a, float b) {
+#ifdef __CUDA_ARCH__
+  return __fmul_rn(a, b);
+#else
+  return a * b;
+#endif
+}
 // a * b = p + e exactly
 PPE_HD df two_prod(float a, float b) {
-  const float p = a * b;
+  const float p = mul_rn(a, b);
   const float e = fmaf(a, b, -p);
   return {p, e};
 }
@@ -195,23 +205,32 @@ PPE_HD df df_recipz(df a) {
   return {y0, y0 * e};
 }
 
+// max(a + b, 0) on signed integers (one instruction on the device)
+PPE_HD int addmax0(int a, int b) {
+#ifdef __CUDA_ARCH__
+  return __viaddmax_s32(a, b, 0);
+#else
+  return a + b > 0 ? a + b : 0;
+#endif
+}
+
 // IEEE double -> pair (see header comment).  Relative error <= 2^-48.
-// hi: the 9 bits below the sign of (hw << 3 | lw >> 29) hold the exponent
-// modulo 512 and the top 23 mantissa bits follow, so adding 128 << 23
-// rebiases 1023 -> 127 (modulo 512) for every in-range exponent and the sign
-// is or-ed back.  lo: the 29 low mantissa bits, converted once, times
-// 2^(e - 1075) = 2^(E_hi - 52), whose bit pattern (with the sign of x) is hi's
-// sign and exponent field minus 52 << 23.  |x| < 2^-74 gives (0, 0).
+// hi: the magnitude's high word less 896 << 20 rebiases the exponent 1023 ->
+// 127 (clamped at zero for |x| < 2^-127); shifted left by three with the top
+// three bits of the low word it is the float's exponent and 23 mantissa bits,
+// and the sign is or-ed back.  lo: the 29 low mantissa bits, converted once,
+// times 2^-52 and times the signed power of two of hi (hi's sign and exponent
+// field).  Nine operations instead of the twelve of a form that tested the
+// range and selected zeros (they are a quarter of the right-hand side's
+// instructions); zeros keep their sign and a zero low part.
 PPE_HD df d2df(double x) {
   const uint64_t b = d_bits(x);
   const uint32_t hw = (uint32_t)(b >> 32), lw = (uint32_t)b;
-  const uint32_t hb = (((hw << 3) | (lw >> 29)) + 0x40000000u) | (hw & 0x80000000u);
-  const float sc = f_from((hb & 0xFF800000u) - 0x1A000000u);
-  const float lo = (float)(lw & 0x1FFFFFFFu) * sc;
-  const bool ok = (hw & 0x7FF00000u) >= (949u << 20);
+  const uint32_t m = (uint32_t)addmax0((int)(hw & 0x7FFFFFFFu), -(896 << 20));
+  const uint32_t hb = ((m << 3) | (lw >> 29)) | (hw & 0x80000000u);
   df r;
-  r.hi = ok ? f_from(hb) : 0.0f;
-  r.lo = ok ? lo : 0.0f;
+  r.hi = f_from(hb);
+  r.lo = ((float)(lw & 0x1FFFFFFFu) * 0x1p-52f) * f_from(hb & 0xFF800000u);
   return r;
 }
 

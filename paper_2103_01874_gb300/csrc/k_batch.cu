@@ -131,7 +131,10 @@ unsigned batch_stage_chunk(int nx, int ny, int nz, int stage, long grain) {
 }
 
 size_t batch_smem(int nx, int ny, int nz) {
-  size_t m = rhs_smem(nx, kBatchRhsLines);
+  // the right-hand side's rows (256 / nx stacks per CTA, two halo lines) and raw slots
+  const size_t tj = (size_t)(kRhsThreads / nx) * kBatchRhsLines;
+  size_t m = sizeof(df) * (size_t)nx * (2 * (tj + 2) + tj) +
+             (rhs_slots_in_smem(kBatchRhsLines) ? sizeof(double) * rhs_slots(kBatchRhsLines, 2) * kRhsThreads : 0);
   const int lx = (int)lines_per_tile(nx / 2, batch_lpb(nx));
   m = std::max(m, pow2(nx / 2) ? xrg_smem(nx, lx) : xfwd_smem<float>(nx, lx));
   m = std::max(m, pow2(nx / 2) ? xrg_smem(nx, lx) : xinv_smem<float>(nx, lx));

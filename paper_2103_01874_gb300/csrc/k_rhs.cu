@@ -3,26 +3,26 @@
 //   f = D[beta_f G p_hat] + (rho_0/dt)(D u* - S),  beta_f = 1 - rho_0/rho_f,
 //   p_hat = 2 p^n - p^{n-1}                                        (Eq. (32))
 //
-// Written per face as Q~_f = beta_f (p_hat_R - p_hat_L) + (rho_0/dt) h u*_f (h
-// the spacing of the face's direction), so that f = sum_dir (Q~_+ - Q~_-)/h^2
-// - (rho_0/dt) S.  The same face quantity also gives the explicitly
-// split velocity of Eq. (33):  since 1/rho_f - 1/rho_0 = -beta_f/rho_0,
-//   u^{n+1}_f = u*_f + (dt/rho_0) beta_f (G p_hat)_f - (dt/rho_0) (G p^{n+1})_f
-// and this kernel stores u_pre_f = u*_f + (dt/rho_0) beta_f (G p_hat)_f, leaving
-// only the pressure-gradient term for the kernel that runs after the solve.
+// Written per face as u_pre_f = u*_f + (dt/rho_0) beta_f (G p_hat)_f, the explicitly
+// split velocity of Eq. (33) (since 1/rho_f - 1/rho_0 = -beta_f/rho_0,
+// u^{n+1}_f = u_pre_f - (dt/rho_0) (G p^{n+1})_f), so that
+//   f = (rho_0/dt) (D u_pre - S).
+// This kernel stores u_pre and f, leaving only the pressure-gradient term for
+// the kernel that runs after the solve.
 //
 // Arithmetic: p_hat is formed by one FP64 fused multiply-add; it and the other
 // FP64 inputs are split into float pairs with integer operations (dfloat.cuh)
 // and every face and cell value is formed in pair arithmetic.
 //
 // Blocking: a CTA owns `tj` consecutive y-lines for a chunk of `kc` z-planes and
-// marches upward in z.  Each thread owns fixed (i, j) columns of the tile and
-// keeps in registers the next plane's p_hat and rho and the value of the lower
-// z face of its cells; shared memory holds the current plane's p_hat and rho
-// (the tj lines plus one halo line on each side) and the x- and y-face values.
-// Each input value is converted once per CTA (plus halo lines), each face is
-// evaluated once.  f is written as float pairs (the forward x transform reads
-// it back, k_xfwd) and/or as FP64.
+// marches upward in z.  Grids up to 512 wide take the column-stack form
+// (rhs.cuh), wider ones the general march below: each thread owns fixed (i, j)
+// columns of the tile and keeps in registers the next plane's p_hat and rho
+// and the value of the lower z face of its cells; shared memory holds the
+// current plane's p_hat and rho (the tj lines plus one halo line on each side)
+// and the x- and y-face values.  Each input value is converted once per CTA
+// (plus halo lines), each face is evaluated once.  f is written as float pairs
+// (the forward x transform reads it back, k_xfwd) and/or as FP64.
 #include "dfloat.cuh"
 #include "ppe_internal.h"
 #include "pdl.cuh"
@@ -36,7 +36,7 @@ namespace ppe {
 // and u_pre, v_pre, w_pre always written, f as FP64 when given) or, with
 // PROJ = false, f as FP64 only (ppe_rhs)
 template <int CPT, int RULE, bool PROJ>
-__global__ void __launch_bounds__(kRhsThreads, (CPT <= 2) ? 3 : (CPT == 4 ? 2 : 1))
+__global__ void __launch_bounds__(kRhsThreads, CPT == 4 ? 2 : 1)
     k_rhs_march(GridDev g, StencilIn in, DevScalars* sc, RhsOut out, int tj, int kc) {
   pdl_enter();
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -46,7 +46,6 @@ __global__ void __launch_bounds__(kRhsThreads, (CPT <= 2) ? 3 : (CPT == 4 ? 2 : 
   const int j0 = jt * tj, k0 = kci * kc;
   const int steps = min(kc, nz - k0);
   const int nl = tj + 2;  // lines of the current plane held in shared memory (with halos)
-  constexpr int rule = RULE;
 
   // shared: current plane p_hat and rho (nl lines), x-face and y-face values
   df* P = reinterpret_cast<df*>(smem_raw);  // [nl][nx]
@@ -76,6 +75,10 @@ __global__ void __launch_bounds__(kRhsThreads, (CPT <= 2) ? 3 : (CPT == 4 ? 2 : 
   auto cell = [&](int kk, int j, int i) -> uint32_t { return (uint32_t)kk * plane + (uint32_t)(j * nx + i); };
   auto wrapk = [&](int kk) { return kk < 0 ? kk + nz : (kk >= nz ? kk - nz : kk); };  // kk in [-nz, 2 nz)
 
+  auto face = [&](df rl, df rh, df pl, df ph, df us, df gh) {
+    return face_upre<RULE, false>(rl, rh, pl, ph, us, gh, K);
+  };
+
   // own columns of plane kk into (pv, rv)
   auto load_cols = [&](int kk, df* pv, df* rv) {
     kk = wrapk(kk);
@@ -93,7 +96,7 @@ __global__ void __launch_bounds__(kRhsThreads, (CPT <= 2) ? 3 : (CPT == 4 ? 2 : 
 #pragma unroll
     for (int u = 0; u < CPT; ++u) {
       pv[u] = phat_of(a[u], b[u]);  // p_hat = 2 p^n - p^{n-1}
-      rv[u] = d2df(r[u]);
+      rv[u] = rho_cell<RULE>(d2df(r[u]), K);
     }
   };
   // halo lines j0-1 and j0+tj of plane kk into shared lines 0 and nl-1
@@ -107,7 +110,7 @@ __global__ void __launch_bounds__(kRhsThreads, (CPT <= 2) ? 3 : (CPT == 4 ? 2 : 
       if (j >= 0 && j < ny) {
         const uint32_t c = cell(kk, j, i);
         pv = phat_of(__ldg(in.pn + c), __ldg(in.pnm1 + c));
-        rv = d2df(__ldg(in.rho + c));
+        rv = rho_cell<RULE>(d2df(__ldg(in.rho + c)), K);
       }
       P[l * nx + i] = pv;
       R[l * nx + i] = rv;
@@ -123,9 +126,8 @@ __global__ void __launch_bounds__(kRhsThreads, (CPT <= 2) ? 3 : (CPT == 4 ? 2 : 
     for (int u = 0; u < CPT; ++u) {
       q[u] = {0.0f, 0.0f};
       if (!cv[u]) continue;
-      const FaceOut fo = face_q(rl[u], rh[u], pl[u], ph[u], d2df(ws[u]), K.cz, K.gz, K, rule);
-      q[u] = fo.q;
-      if (PROJ && owned) out.wpre[cell(kf, j0 + cj[u], ci[u])] = fo.upre;
+      q[u] = face(rl[u], rh[u], pl[u], ph[u], d2df(ws[u]), K.gz);
+      if (PROJ && owned) out.wpre[cell(kf, j0 + cj[u], ci[u])] = q[u];
     }
   };
 
@@ -188,9 +190,8 @@ __global__ void __launch_bounds__(kRhsThreads, (CPT <= 2) ? 3 : (CPT == 4 ? 2 : 
       if (cv[u]) {
         const int r = (cj[u] + 1) * nx;
         const int i = ci[u], im = (i == 0) ? nx - 1 : i - 1;
-        const FaceOut fo = face_q(R[r + im], R[r + i], P[r + im], P[r + i], d2df(us_[u]), K.cx, K.gx, K, rule);
-        q = fo.q;
-        if (PROJ) out.upre[cell(k, j0 + cj[u], i)] = fo.upre;
+        q = face(R[r + im], R[r + i], P[r + im], P[r + i], d2df(us_[u]), K.gx);
+        if (PROJ) out.upre[cell(k, j0 + cj[u], i)] = q;
       }
       QX[cj[u] * nx + ci[u]] = q;
     }
@@ -219,20 +220,16 @@ __global__ void __launch_bounds__(kRhsThreads, (CPT <= 2) ? 3 : (CPT == 4 ? 2 : 
             const bool own = (jf < tj) || (j == ny);
             if (j == ny && g.top_open) {  // open top: p = 0 on the face, ghost -p_hat above
               const int rl = jf * nx + i;
-              const FaceOut fo = face_q(R[rl], R[rl], P[rl], df_neg(P[rl]), vs, K.cy, K.gy, K, rule);
-              q = fo.q;
-              if (PROJ && own) out.vpre[cvv] = fo.upre;
-            } else if (j == 0 || j == ny) {  // wall
-              q = df_norm(df_mulz(K.cy, vs));
-              if (PROJ && own) out.vpre[cvv] = vs;
+              q = face(R[rl], R[rl], P[rl], df_neg(P[rl]), vs, K.gy);
+            } else if (j == 0 || j == ny) {  // wall: u_pre = v*
+              q = vs;
               wsum = (j == ny) ? df_addz(wsum, vs) : df_subz(wsum, vs);
               wmax = fmaxf(wmax, fabsf(vs.hi));
             } else {
               const int rl = jf * nx + i, rh = (jf + 1) * nx + i;
-              const FaceOut fo = face_q(R[rl], R[rh], P[rl], P[rh], vs, K.cy, K.gy, K, rule);
-              q = fo.q;
-              if (PROJ && own) out.vpre[cvv] = fo.upre;
+              q = face(R[rl], R[rh], P[rl], P[rh], vs, K.gy);
             }
+            if (PROJ && own) out.vpre[cvv] = q;
           }
           QY[idx] = q;
         }
@@ -244,9 +241,8 @@ __global__ void __launch_bounds__(kRhsThreads, (CPT <= 2) ? 3 : (CPT == 4 ? 2 : 
       QZup[u] = {0.0f, 0.0f};
       if (!cv[u]) continue;
       const int r = (cj[u] + 1) * nx + ci[u];
-      const FaceOut fo = face_q(R[r], R1[u], P[r], P1[u], d2df(ws_[u]), K.cz, K.gz, K, rule);
-      QZup[u] = fo.q;
-      if (PROJ && k + 1 < k0 + steps) out.wpre[cell(wrapk(k + 1), j0 + cj[u], ci[u])] = fo.upre;
+      QZup[u] = face(R[r], R1[u], P[r], P1[u], d2df(ws_[u]), K.gz);
+      if (PROJ && k + 1 < k0 + steps) out.wpre[cell(wrapk(k + 1), j0 + cj[u], ci[u])] = QZup[u];
     }
     __syncthreads();
     // ---- phase B: cells of plane k
@@ -255,10 +251,10 @@ __global__ void __launch_bounds__(kRhsThreads, (CPT <= 2) ? 3 : (CPT == 4 ? 2 : 
       if (!cv[u]) continue;
       const int i = ci[u], jj = cj[u];
       const int ip = (i + 1 == nx) ? 0 : i + 1;
-      // f = sum over directions of (Q~_+ - Q~_-) / h^2 - (rho_0/dt) S
-      const df dxq = df_mulz(df_subz(QX[jj * nx + ip], QX[jj * nx + i]), K.lx);
-      const df dyq = df_mulz(df_subz(QY[(jj + 1) * nx + i], QY[jj * nx + i]), K.ly);
-      const df dzq = df_mulz(df_subz(QZup[u], QZ[u]), K.lz);
+      // f = (rho_0/dt) (D u_pre - S)
+      const df dxq = df_mulz(df_subz(QX[jj * nx + ip], QX[jj * nx + i]), K.cx);
+      const df dyq = df_mulz(df_subz(QY[(jj + 1) * nx + i], QY[jj * nx + i]), K.cy);
+      const df dzq = df_mulz(df_subz(QZup[u], QZ[u]), K.cz);
       const uint32_t c = cell(k, j0 + jj, i);
       const df sv = d2df(ss_[u]);
       const df f = df_norm(df_subz(df_addz(df_addz(dxq, dyq), dzq), df_mulz(K.c, sv)));
@@ -282,7 +278,7 @@ __global__ void __launch_bounds__(kRhsThreads, (CPT <= 2) ? 3 : (CPT == 4 ? 2 : 
 #pragma unroll
       for (int u = 0; u < CPT; ++u) {
         P1[u] = phat_of(rp[u], rm[u]);
-        R1[u] = d2df(rr[u]);
+        R1[u] = rho_cell<RULE>(d2df(rr[u]), K);
       }
       __syncthreads();
     }
@@ -301,22 +297,73 @@ __global__ void __launch_bounds__(kRhsThreads, (CPT <= 2) ? 3 : (CPT == 4 ? 2 : 
 
 __global__ void k_finish_sums(GridDev g, DevScalars* sc) { finish_sums(sc, g); }
 
-// Column-stack form of the march (rhs.cuh): one CTA per tile.
-template <int S, int RULE, bool PROJ>
-__global__ void __launch_bounds__(kRhsThreads, (S <= 2) ? 3 : (S == 4 ? 2 : 1))
+// Column-stack form of the march (rhs.cuh): one CTA of BT threads at most per
+// tile.  What bounds it: instruction issue and the latency of a step's loads
+// (493 warp instructions per 32 cells, 683 before; raw values prefetched into
+// shared memory, whole stacks per CTA).  256^3, projection outputs: 371 -> 305
+// us (1.61 GB moved, 5.3 TB/s); 384 x 256 x 384 (the general march before):
+// 1248 -> 690; 192^3 (a quarter of the threads idle before): 201 -> 132; 128^3:
+// 66 -> 45.  The register budget (80 a thread for S <= 2: three CTAs of 256 threads
+// or two of 384 per SM) keeps the loads of the next plane in flight; a CTA of
+// up to 512 threads runs alone on its SM.
+template <int S, int RULE, bool PROJ, int BT, int NXC>
+__global__ void __launch_bounds__(BT, BT == 256 ? (S <= 2 ? 3 : (S == 4 ? 2 : 1)) : (BT == 384 && S <= 2 ? 2 : 1))
     k_rhs_stack(GridDev g, StencilIn in, DevScalars* sc, RhsOut out, int kc) {
   pdl_enter();
-  rhs_stack_tile<S, RULE, PROJ>(g, in, sc, out, kc, blockIdx.x);
+  rhs_stack_tile<S, RULE, PROJ, NXC>(g, in, sc, out, kc, blockIdx.x);
 }
 
-// Lines per tile: the stack form (nx <= 256) has 256 / nx stacks of `lines`
-// lines each; the general form has `lines` lines.
-int rhs_tile_lines(int nx, int lines) { return nx <= kRhsThreads ? (kRhsThreads / nx) * lines : lines; }
 
-size_t rhs_smem(int nx, int lines) {
-  const size_t tj = rhs_tile_lines(nx, lines), nl = tj + 2;
-  if (nx <= kRhsThreads) return sizeof(df) * (2 * nl * nx + tj * nx);
+namespace {
+// Stacks of a launch: those that fill its grid best, within the block bound of
+// the instance of this nx (two at least where it gives a thread one halo cell).
+int launch_stacks(int nx, int ny, int S) {
+  const int s0 = stacks_of(nx);
+  return stacks_of(nx, ny, S, s0 > 1 ? 2 : 1, stack_bound(stack_threads(nx, s0)));
+}
+size_t stack_smem(int nx, int stacks, int S) {
+  const size_t tj = (size_t)stacks * S, nl = tj + 2;
+  return sizeof(df) * (2 * nl * nx + tj * nx) +
+         (rhs_slots_in_smem(S) ? sizeof(double) * rhs_slots(S, 2) * stack_threads(nx, stacks) : 0);
+}
+}  // namespace
+
+// Lines per tile: the stack form (nx <= 512) has launch_stacks stacks of
+// `lines` lines each; the general form has `lines` lines.
+int rhs_tile_lines(int nx, int ny, int lines) {
+  return nx <= kRhsStackNx ? launch_stacks(nx, ny, lines) * lines : lines;
+}
+
+size_t rhs_smem(int nx, int ny, int lines) {
+  if (nx <= kRhsStackNx) return stack_smem(nx, launch_stacks(nx, ny, lines), lines);
+  const size_t tj = lines, nl = tj + 2;
   return sizeof(df) * (2 * nl * nx + tj * nx + (tj + 1) * nx);
+}
+
+// Planes per CTA of the column-stack form at S = 2.  A CTA marches kc planes
+// after a prologue worth about one and a half; with N CTAs on `slots` resident
+// places the march takes (N / slots + 1/2) (kc + 3/2) steps, and where one wave
+// holds them all, kc + 3/2 steps that are the shorter the emptier the SMs
+// (measured over kc = 1 .. 32 at 32^3 .. 384 x 256 x 384: within 4 % of the best
+// of each, except 12 % on 48 x 192 x 32; the fixed kc = 8 before cost 32^3 24
+// instead of 10 us, 64^3 24 instead of 14).
+int rhs_planes(int nx, int ny, int nz) {
+  if (nx > kRhsStackNx) return nz < 8 ? nz : 8;
+  const int stacks = launch_stacks(nx, ny, 2), threads = stack_threads(nx, stacks);
+  const int bound = stack_bound(threads);
+  const double slots = 152.0 * (bound == 512 ? 1 : 65536 / (80 * threads));
+  const int ntile = (ny + 2 * stacks - 1) / (2 * stacks);
+  int best = 1;
+  double least = 0.0;
+  for (int kc = 1; kc <= 12 && kc <= nz; ++kc) {
+    const double w = ntile * ((nz + kc - 1) / kc) / slots;
+    const double t = (w <= 1.0 ? 0.45 + 0.55 * w : w + 0.5) * (kc + 1.5);
+    if (kc == 1 || t < least) {
+      least = t;
+      best = kc;
+    }
+  }
+  return best;
 }
 
 int rhs_max_lines(int nx) {
@@ -326,6 +373,39 @@ int rhs_max_lines(int nx) {
   return tj;
 }
 
+namespace {
+// Calls f(kernel) with the column-stack instance for (S, rule, proj, nx).
+// The projection's default S = 2 has instances with nx compiled in for the
+// usual widths (their CTAs are whole stacks: threads = stacks * nx).
+template <int S, int RULE, bool PROJ, class F>
+void stack_instance(int nx, int threads, F&& f) {
+  if constexpr (S == 2 && PROJ) {
+#define PPE_NX(N) \
+    case N: return f(k_rhs_stack<2, RULE, true, stack_bound(stack_threads(N, stacks_of(N))), N>);
+    switch (nx) {
+      PPE_NX(32) PPE_NX(64) PPE_NX(96) PPE_NX(128) PPE_NX(192) PPE_NX(256) PPE_NX(384)
+      default: break;
+    }
+#undef PPE_NX
+  }
+  if (threads <= 256) return f(k_rhs_stack<S, RULE, PROJ, 256, 0>);
+  if constexpr (S <= 2)
+    if (threads <= 384) return f(k_rhs_stack<S, RULE, PROJ, 384, 0>);
+  f(k_rhs_stack<S, RULE, PROJ, 512, 0>);
+}
+
+template <int S, class F>
+void stack_kernel(int nx, int threads, int rule, bool proj, F&& f) {
+  if (rule == 0) {
+    if (proj) stack_instance<S, 0, true>(nx, threads, f);
+    else stack_instance<S, 0, false>(nx, threads, f);
+  } else {
+    if (proj) stack_instance<S, 1, true>(nx, threads, f);
+    else stack_instance<S, 1, false>(nx, threads, f);
+  }
+}
+}  // namespace
+
 cudaError_t launch_rhs(const GridDev& g, const StencilIn& in, DevScalars* sc, double* f64, df* fdf, df* upre,
                        df* vpre, df* wpre, int tj, int kc, cudaStream_t st) {
   RhsOut o;
@@ -334,34 +414,28 @@ cudaError_t launch_rhs(const GridDev& g, const StencilIn& in, DevScalars* sc, do
   o.upre = upre;
   o.vpre = vpre;
   o.wpre = wpre;
-  const int tile = rhs_tile_lines(g.nx, tj);
+  const int tile = rhs_tile_lines(g.nx, g.ny, tj);
   const int ntile = (g.ny + tile - 1) / tile;
   const int nchunk = (g.nz + kc - 1) / kc;
-  const size_t sm = rhs_smem(g.nx, tj);
+  const size_t sm = rhs_smem(g.nx, g.ny, tj);
   const int grid = ntile * nchunk;
   const bool proj = fdf != nullptr;
   if (proj && !(upre && vpre && wpre)) return cudaErrorInvalidValue;
   if (!proj && !f64) return cudaErrorInvalidValue;
-  if (g.nx <= kRhsThreads) {
+  if (g.nx <= kRhsStackNx) {
     // column-stack form: tj is the stack height S
-    auto go = [&](auto kernel) { launch_pdl(kernel, grid, kRhsThreads, sm, st, g, in, sc, o, kc); };
-#define PPE_STACK_CASE(C)                                                        \
-    if (tj == C) {                                                               \
-      if (in.face_rule == 0) {                                                   \
-        if (proj) go(k_rhs_stack<C, 0, true>); else go(k_rhs_stack<C, 0, false>); \
-      } else {                                                                   \
-        if (proj) go(k_rhs_stack<C, 1, true>); else go(k_rhs_stack<C, 1, false>); \
-      }                                                                          \
+    const int threads = stack_threads(g.nx, launch_stacks(g.nx, g.ny, tj));
+    auto go = [&](auto kernel) { launch_pdl(kernel, grid, threads, sm, st, g, in, sc, o, kc); };
+    switch (tj) {
+      case 1: stack_kernel<1>(g.nx, threads, in.face_rule, proj, go); break;
+      case 2: stack_kernel<2>(g.nx, threads, in.face_rule, proj, go); break;
+      case 4: stack_kernel<4>(g.nx, threads, in.face_rule, proj, go); break;
+      case 8: stack_kernel<8>(g.nx, threads, in.face_rule, proj, go); break;
+      default: return cudaErrorInvalidValue;
     }
-    PPE_STACK_CASE(1)
-    PPE_STACK_CASE(2)
-    PPE_STACK_CASE(4)
-    PPE_STACK_CASE(8)
-#undef PPE_STACK_CASE
     return cudaGetLastError();
   }
-  const int ncol = tj * g.nx;
-  const int cpt = ncol <= kRhsThreads ? 1 : ncol <= 2 * kRhsThreads ? 2 : ncol <= 4 * kRhsThreads ? 4 : 8;
+  const int cpt = tj * g.nx <= 4 * kRhsThreads ? 4 : 8;
   auto go = [&](auto kernel) { launch_pdl(kernel, grid, kRhsThreads, sm, st, g, in, sc, o, tj, kc); };
   // instance table: [cpt][rule][proj]
 #define PPE_RHS_CASE(C)                                                        \
@@ -372,8 +446,6 @@ cudaError_t launch_rhs(const GridDev& g, const StencilIn& in, DevScalars* sc, do
       if (proj) go(k_rhs_march<C, 1, true>); else go(k_rhs_march<C, 1, false>); \
     }                                                                          \
   }
-  PPE_RHS_CASE(1)
-  PPE_RHS_CASE(2)
   PPE_RHS_CASE(4)
   PPE_RHS_CASE(8)
 #undef PPE_RHS_CASE
@@ -399,34 +471,50 @@ cudaError_t launch_finish_sums(const GridDev& g, DevScalars* sc, cudaStream_t st
   return cudaGetLastError();
 }
 
+namespace {
 template <int C>
-cudaError_t raise_rhs(size_t* cap) {
+cudaError_t raise_march(size_t* cap) {
   cudaError_t e = raise_smem(k_rhs_march<C, 0, true>, cap);
   if (e == cudaSuccess) e = raise_smem(k_rhs_march<C, 0, false>, cap);
   if (e == cudaSuccess) e = raise_smem(k_rhs_march<C, 1, true>, cap);
   if (e == cudaSuccess) e = raise_smem(k_rhs_march<C, 1, false>, cap);
-  if (e == cudaSuccess) e = raise_smem(k_rhs_stack<C, 0, true>, cap);
-  if (e == cudaSuccess) e = raise_smem(k_rhs_stack<C, 0, false>, cap);
-  if (e == cudaSuccess) e = raise_smem(k_rhs_stack<C, 1, true>, cap);
-  if (e == cudaSuccess) e = raise_smem(k_rhs_stack<C, 1, false>, cap);
   return e;
 }
+template <int S>
+cudaError_t raise_stack(size_t* cap) {
+  cudaError_t e = cudaSuccess;
+  auto up = [&](auto kernel) {
+    if (e == cudaSuccess) e = raise_smem(kernel, cap);
+  };
+  // every width with an instance of its own, and one thread count per block bound
+  for (int rule = 0; rule < 2; ++rule) {
+    for (int nx : {32, 64, 96, 128, 192, 256, 384}) stack_kernel<S>(nx, 256, rule, true, up);
+    for (int threads : {256, 384, 512}) {
+      stack_kernel<S>(8, threads, rule, true, up);
+      stack_kernel<S>(8, threads, rule, false, up);
+    }
+  }
+  return e;
+}
+cudaError_t raise_all(size_t* cap) {
+  cudaError_t e = raise_march<4>(cap);
+  if (e == cudaSuccess) e = raise_march<8>(cap);
+  if (e == cudaSuccess) e = raise_stack<1>(cap);
+  if (e == cudaSuccess) e = raise_stack<2>(cap);
+  if (e == cudaSuccess) e = raise_stack<4>(cap);
+  if (e == cudaSuccess) e = raise_stack<8>(cap);
+  return e;
+}
+}  // namespace
 
 cudaError_t set_rhs_smem_limit() {
   size_t cap = kSmemPerCta;
-  cudaError_t e = raise_rhs<1>(&cap);
-  if (e == cudaSuccess) e = raise_rhs<2>(&cap);
-  if (e == cudaSuccess) e = raise_rhs<4>(&cap);
-  if (e == cudaSuccess) e = raise_rhs<8>(&cap);
-  return e;
+  return raise_all(&cap);
 }
 
 size_t rhs_smem_limit() {
   size_t cap = kSmemPerCta;
-  if (raise_rhs<1>(&cap) != cudaSuccess || raise_rhs<2>(&cap) != cudaSuccess || raise_rhs<4>(&cap) != cudaSuccess ||
-      raise_rhs<8>(&cap) != cudaSuccess)
-    return 0;
-  return cap;
+  return raise_all(&cap) == cudaSuccess ? cap : 0;
 }
 
 }  // namespace ppe

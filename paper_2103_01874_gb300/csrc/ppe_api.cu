@@ -769,14 +769,14 @@ bool p32_ok(const ppe_grid& g, const ppe_options& o) {
          (s & (s - 1u)) == 0u;
 }
 
-// Tile sizes of the right-hand-side kernel: largest tj in {8, 4, 2, 1} whose
-// shared memory lets two CTAs share an SM, else one.
+// Tile sizes of the right-hand-side kernel: two lines per stack where a CTA's
+// shared memory allows it, else one.
 void choose_rhs_tiles(ppe_plan_t P) {
   const int nx = P->g.nx;
   int tj = 2;  // measured best at 256^3 on a GB300 (register-limited occupancy)
-  while (tj > 1 && (rhs_smem(nx, tj) > 110 * 1024 || tj > rhs_max_lines(nx))) tj /= 2;
+  while (tj > 1 && (rhs_smem(nx, P->g.ny, tj) > 200 * 1024 || tj > rhs_max_lines(nx))) tj /= 2;
   P->tj = tj;
-  P->kc = P->g.nz < 8 ? P->g.nz : 8;
+  P->kc = rhs_planes(nx, P->g.ny, P->g.nz);
 }
 
 }  // namespace
@@ -1024,7 +1024,7 @@ ppe_status ppe_set_tuning(ppe_plan_t P, const ppe_tuning* t) {
   auto pow2 = [](int v, int lo, int hi) { return v >= lo && v <= hi && (v & (v - 1)) == 0; };
   const size_t lim = 227 * 1024;
   const int nx = P->g.nx, ny = P->g.ny, nz = P->g.nz;
-  if (!pow2(t->rhs_lines, 1, 8) || rhs_smem(nx, t->rhs_lines) > rhs_smem_limit() ||
+  if (!pow2(t->rhs_lines, 1, 8) || rhs_smem(nx, ny, t->rhs_lines) > rhs_smem_limit() ||
       t->rhs_lines > rhs_max_lines(nx))
     return PPE_ERR_INVALID_ARG;
   if (t->rhs_planes < 1 || t->rhs_planes > nz) return PPE_ERR_INVALID_ARG;
@@ -1100,6 +1100,7 @@ ppe_status ppe_rhs(ppe_plan_t P, const double* u, const double* v, const double*
   NvtxRange _nvtx("ppe_rhs");
   if (!P || !u || !v || !w || !S || !rho || !p_n || !p_nm1 || !f || !(dt > 0)) return PPE_ERR_INVALID_ARG;
   StencilIn in = make_in(P, u, v, w, S, rho, p_n, p_nm1, dt);
+  in.min_rho0 = !(rho0 > 0);
   const size_t n = (size_t)P->g.nx * P->g.ny * P->g.nz;
   PPE_LAUNCH(P, K_INIT, launch_init_scalars(P->sc, rho0, P->opt.refine_tol, 0, P->stream));
   if (!(rho0 > 0)) PPE_LAUNCH(P, K_RHO_MIN, launch_rho_min(rho, n, P->sc, P->stream));
@@ -1155,6 +1156,7 @@ ppe_status ppe_project(ppe_plan_t P, const ppe_fields* F) {
       !F->v_out || !F->w_out || !(F->dt > 0))
     return PPE_ERR_INVALID_ARG;
   StencilIn in = make_in(P, F->u, F->v, F->w, F->S, F->rho, F->p_n, F->p_nm1, F->dt);
+  in.min_rho0 = !(F->rho0 > 0);
   const size_t n = (size_t)P->g.nx * P->g.ny * P->g.nz;
   PPE_LAUNCH(P, K_INIT, P->fp32 ? launch_init_scalars(P->sc, F->rho0, P->opt.refine_tol, 0, P->stream, F->p,
                                                        F->u_out, F->v_out, F->w_out)
@@ -1318,6 +1320,7 @@ ppe_status batch_persistent(ppe_batch_t B, int n, const ppe_plan_t* plans, const
     memset(&G, 0, sizeof(G));
     G.g = P->gd;
     G.in = make_in(P, F->u, F->v, F->w, F->S, F->rho, F->p_n, F->p_nm1, F->dt);
+    G.in.min_rho0 = !(F->rho0 > 0);
     G.sc = P->sc;
     G.f64 = F->f;
     G.fdf = P->fdf;

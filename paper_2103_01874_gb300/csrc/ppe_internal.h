@@ -23,7 +23,7 @@ struct StencilConst {
   df idx, idy, idz;
   df gx, gy, gz;   // (dt/rho_0) / dx, ...
   df lx, ly, lz;   // 1/dx^2, 1/dy^2, 1/dz^2
-  df cx, cy, cz;   // (rho_0/dt) dx, (rho_0/dt) dy, (rho_0/dt) dz
+  df cx, cy, cz;   // (rho_0/dt) / dx, ...
 };
 
 // Device-resident scalars of one plan.  Non-negative doubles are kept as their
@@ -104,6 +104,7 @@ struct StencilIn {
   double inv_dt;
   double dt;
   int face_rule;     // 0 arithmetic, 1 harmonic
+  int min_rho0;      // rho_0 is the minimum of rho (not given by the caller)
 };
 
 enum XSource { SRC_F = 1, SRC_RESID = 2, SRC_FDF = 3 };
@@ -115,8 +116,10 @@ cudaError_t launch_rhs(const GridDev& g, const StencilIn& in, DevScalars* sc, do
 // Totals of the per-CTA partial sums into sc (one CTA, finish_sums); the first
 // forward z pass after an x transform of f does the same in its CTA 0.
 cudaError_t launch_finish_sums(const GridDev& g, DevScalars* sc, cudaStream_t st);
-size_t rhs_smem(int nx, int lines);  // dynamic shared memory of the RHS kernel for a rhs_lines value
-int rhs_max_lines(int nx);  // largest rhs_lines value (lines per thread stack, or per tile when nx > 256)
+size_t rhs_smem(int nx, int ny, int lines);  // dynamic shared memory of the RHS kernel for a rhs_lines value
+int rhs_tile_lines(int nx, int ny, int lines);  // lines per CTA
+int rhs_planes(int nx, int ny, int nz);         // z planes per CTA, chosen for the grid
+int rhs_max_lines(int nx);  // largest rhs_lines value (lines per thread stack, or per tile when nx > 512)
 cudaError_t set_rhs_smem_limit();
 size_t rhs_smem_limit();  // largest dynamic shared memory every k_rhs_march instance accepts
 constexpr size_t kSmemPerCta = 227 * 1024;  // opt-in shared memory per CTA (static + dynamic)

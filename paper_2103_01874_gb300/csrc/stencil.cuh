@@ -37,9 +37,9 @@ __device__ __forceinline__ StencilConst make_const(const GridDev& g, double rho0
   K.lx = d2df(g.idx * g.idx);
   K.ly = d2df(g.idy * g.idy);
   K.lz = d2df(g.idz * g.idz);
-  K.cx = d2df(rho0 / dt / g.idx);
-  K.cy = d2df(rho0 / dt / g.idy);
-  K.cz = d2df(rho0 / dt / g.idz);
+  K.cx = d2df(rho0 / dt * g.idx);
+  K.cy = d2df(rho0 / dt * g.idy);
+  K.cz = d2df(rho0 / dt * g.idz);
   return K;
 }
 
@@ -51,28 +51,52 @@ __device__ __forceinline__ df beta_df(df a, df b, const StencilConst& K, int rul
   return df_subz(one, df_mulz(K.r0h, df_addz(df_recipz(a), df_recipz(b))));        // 1 - (rho_0/2)(1/a+1/b)
 }
 
-// Split flux of one face without the 1/h factor, Q~ = beta_f (p_hat_R - p_hat_L)
-// + (rho_0/dt) h u*_f, and the explicitly split velocity
-// u_pre = u*_f + (dt/rho_0)(1/h) beta_f (p_hat_R - p_hat_L); h the spacing of
-// the face's direction, ch = (rho_0/dt) h, gh = (dt/rho_0)/h.  Since
-// ch gh = 1, u_pre = gh Q~: one product of the flux instead of a product and
-// a sum (the two differ by the pair rounding of the constants, ~1e-14
-// relative, and D u_pre = (dt/rho_0)(f + (rho_0/dt) S) holds either way).
-// Both are left unnormalised (see the lazy operations in dfloat.cuh): every
-// consumer -- the divergence, the correction's subtraction and its exact
-// conversion to FP64 -- takes them through lazy pair operations, and a
-// normalisation only rewrites the same value (about 5 % fewer instructions
-// in the right-hand-side kernels).
-struct FaceOut {
-  df q, upre;
-};
-__device__ __forceinline__ FaceOut face_q(df rl, df rh, df pl, df ph, df us, df ch, df gh, const StencilConst& K,
-                                          int rule) {
-  const df bg = df_mulz(beta_df(rl, rh, K, rule), df_subz(ph, pl));
-  FaceOut o;
-  o.q = df_addz(bg, df_mulz(ch, us));
-  o.upre = df_mulz(gh, o.q);
-  return o;
+// What the right-hand side keeps per cell for the face densities: rho itself
+// (arithmetic rule) or (rho_0/2)/rho (harmonic rule: beta_f is 1 minus the sum
+// of the two cells' values, so the reciprocal is taken once per cell instead
+// of at each of its six faces).
+template <int RULE>
+__device__ __forceinline__ df rho_cell(df rho, const StencilConst& K) {
+  if (RULE == 0) return rho;
+  return df_mulz(K.r0h, df_recipz(rho));
+}
+
+// beta_f = 1 - rho_0/rho_f from two cells' rho_cell values (unnormalised pair).
+// Arithmetic rule: t = 2 rho_0/(a + b) as y + e/(a + b) with y = fl(2 rho_0 rcp(a + b))
+// and e = 2 rho_0 - (a + b) y from two fused multiply-adds (the correction of
+// a quotient by its remainder; relative error that of the seed squared,
+// ~2^-46, as a Newton step's), so neither the reciprocal nor its product with
+// 2 rho_0 is formed as a pair: 17 operations against 26.
+// TAME: rho_0 is the minimum of rho, hence t <= 1 (up to its last bit) and
+// 1 - t needs only the fast two-sum; a rho_0 given by the caller may be larger.
+template <int RULE, bool TAME>
+__device__ __forceinline__ df beta_cells(df a, df b, const StencilConst& K) {
+  const df s = df_addz(a, b);
+  float y, tl;  // t = y + tl
+  if (RULE == 0) {
+    const float rc = rcp_seed(s.hi);
+    y = mul_rn(K.r02.hi, rc);
+    const float e = fmaf(-s.hi, y, K.r02.hi) + fmaf(-s.lo, y, K.r02.lo);
+    tl = mul_rn(e, rc);
+  } else {
+    y = s.hi;
+    tl = s.lo;
+  }
+  const df d = TAME ? fast_two_sum(1.0f, -y) : two_sum(1.0f, -y);
+  return {d.hi, d.lo - tl};
+}
+
+// Explicitly split velocity of one face (Eq. (33) without its G p^{n+1} term),
+//   u_pre = u*_f + (dt/rho_0)(1/h) beta_f (p_hat_R - p_hat_L),  gh = (dt/rho_0)/h.
+// It is also the face quantity of the right-hand side: by Eq. (34)
+//   f = (rho_0/dt) (D u_pre - S),
+// so no separate flux is formed (an earlier form kept Q~ = beta Delta p_hat +
+// (rho_0/dt) h u* and u_pre = gh Q~: one pair product more per face).  Left
+// unnormalised (the lazy operations of dfloat.cuh): the divergence, the
+// correction's subtraction and its conversion to FP64 take it so.
+template <int RULE, bool TAME>
+__device__ __forceinline__ df face_upre(df rl, df rh, df pl, df ph, df us, df gh, const StencilConst& K) {
+  return df_addz(us, df_mulz(df_mulz(beta_cells<RULE, TAME>(rl, rh, K), df_subz(ph, pl)), gh));
 }
 
 // p_hat = 2 p^n - p^{n-1} (Eq. (32)): one FP64 fused multiply-add (a single
