@@ -211,6 +211,67 @@ __device__ __forceinline__ void dft_ct(cpx<T>* v) {
   }
 }
 
+// exp(-+ 2 pi i m / 12) for a compile-time m, times v: multiples of a quarter
+// turn are exact rotations, the others use cos and sin of pi/6 and pi/3.
+template <typename T, bool INV, int M12>
+__device__ __forceinline__ cpx<T> tw12(cpx<T> v) {
+  constexpr int m = ((M12 % 12) + 12) % 12;
+  constexpr double C = 0.86602540378443864676372317075294;  // sqrt(3)/2
+  constexpr double c = (m == 1 || m == 11) ? C : (m == 2 || m == 10) ? 0.5 : (m == 4 || m == 8) ? -0.5 : -C;
+  constexpr double s = (m == 1 || m == 5) ? 0.5 : (m == 2 || m == 4) ? C : (m == 7 || m == 11) ? -0.5 : -C;
+  if (m == 0) return v;
+  if (m == 6) return {-v.x, -v.y};
+  if (m == 3) return rot<T, INV>(v);
+  if (m == 9) return rot<T, !INV>(v);
+  constexpr T cr = (T)c, si = INV ? (T)s : (T)(-s);
+  return {v.x * cr - v.y * si, v.x * si + v.y * cr};
+}
+
+// R = 3 R2 (6 and 12): 3-point DFTs on the stride-R2 subsequences, twiddles
+// w_R^(j2 k1), R2-point DFTs (as dft_ct).
+template <typename T, bool INV, int R2>
+__device__ __forceinline__ void dft_3x(cpx<T>* v) {
+  constexpr int R = 3 * R2;
+  cpx<T> a[R];
+#pragma unroll
+  for (int j2 = 0; j2 < R2; ++j2) {
+    cpx<T> s[3] = {v[j2], v[j2 + R2], v[j2 + 2 * R2]};
+    SmallDft<T, INV, 3>::run(s);
+#pragma unroll
+    for (int k1 = 0; k1 < 3; ++k1) a[j2 * 3 + k1] = s[k1];
+  }
+#pragma unroll
+  for (int j2 = 1; j2 < R2; ++j2) {
+#pragma unroll
+    for (int k1 = 1; k1 < 3; ++k1) {
+      cpx<T>& x = a[j2 * 3 + k1];
+      switch (j2 * k1 * (12 / R)) {  // resolved at compile time after unrolling
+        case 1: x = tw12<T, INV, 1>(x); break;
+        case 2: x = tw12<T, INV, 2>(x); break;
+        case 3: x = tw12<T, INV, 3>(x); break;
+        case 4: x = tw12<T, INV, 4>(x); break;
+        case 6: x = tw12<T, INV, 6>(x); break;
+        default: break;
+      }
+    }
+  }
+#pragma unroll
+  for (int k1 = 0; k1 < 3; ++k1) {
+    cpx<T> s[R2];
+#pragma unroll
+    for (int j2 = 0; j2 < R2; ++j2) s[j2] = a[j2 * 3 + k1];
+    SmallDft<T, INV, R2>::run(s);
+#pragma unroll
+    for (int k2 = 0; k2 < R2; ++k2) v[k1 + 3 * k2] = s[k2];
+  }
+}
+template <typename T, bool INV> struct SmallDft<T, INV, 6> {
+  static __device__ __forceinline__ void run(cpx<T>* v) { dft_3x<T, INV, 2>(v); }
+};
+template <typename T, bool INV> struct SmallDft<T, INV, 12> {
+  static __device__ __forceinline__ void run(cpx<T>* v) { dft_3x<T, INV, 4>(v); }
+};
+
 template <typename T, bool INV> struct SmallDft<T, INV, 8> {
   static __device__ __forceinline__ void run(cpx<T>* v) { dft_ct<T, INV, 2, 4>(v); }
 };
@@ -366,14 +427,22 @@ __device__ __forceinline__ cpx<T>* fft_lines_ct(cpx<T>* a, cpx<T>* b, int nl_log
 
 
 // ---------------------------------------------------------------------------
-// Register-staged variant for power-of-two lengths 16 <= N <= 512 (FP32
-// lines).  Each line is transformed by TPL = N/16 threads; between passes a
-// thread keeps 16 elements in registers, so a pass costs one shared-memory
-// store and one load per element, and there is no separate staging copy: the
-// first pass takes its butterfly inputs from a caller functor `ld(e)` (global
-// memory, values computed on the fly, or the shared buffer) and the last pass
-// hands its outputs to `st(e, v)`.  Radix sequence, twiddles and butterflies
-// are those of fft_lines_ct.
+// Register-staged variant (FP32 lines).  Each line is transformed by a few
+// threads (RegPlan); between passes a thread keeps its butterflies' elements
+// in registers, so a pass costs one shared-memory store and one load per
+// element, and there is no separate staging copy: the first pass takes its
+// butterfly inputs from a caller functor `ld(e)` (global memory, values
+// computed on the fly, or the shared buffer) and the last pass hands its
+// outputs to `st(e, v)`.  Twiddles and butterflies are those of fft_lines_ct.
+//
+// RegPlan<N>: power-of-two lengths 16 .. 512, N/16 threads a line with 16
+// elements each, radices 16, 8, 4, 2.
+// SplitPlan<N>: lengths with a factor 3 (24 .. 384) and the shortest powers of
+// two in two passes (three at 384) of radices 4 .. 16 on as many threads as
+// the pass with the most butterflies has, so that the other pass leaves some
+// idle (6 of 8 at 48, 8 of 12 at 96, 12 of 16 at 192).  At 16 and 32 points
+// (RegPlan: one or two threads a line) it shortens the serial chain of a
+// thread, which is all that the smallest grids wait for.
 //
 // Shared layout: element e of the thread's line at ln[row(e) * es], ln the
 // line's base; row(e) = e + e/16 inserts one padding row every 16 elements,
@@ -401,23 +470,45 @@ __device__ __forceinline__ int rowp(int e) {
   return LAYOUT == PAD_ROWS ? row(e) : (LAYOUT == XOR_ROWS ? (e ^ ((e >> 4) & 15)) : e);
 }
 
+template <int LEN>
+struct RegPlan {
+  static constexpr int N = LEN, T = LEN / 16, passes = ctfft::nst(LEN, 16);
+  static constexpr int radix(int s) { return ctfft::radix_at(LEN, s, 16); }
+  static constexpr int ns(int s) { return ctfft::ns_at(LEN, s, 16); }
+};
+template <int LEN>
+struct SplitPlan {
+  static constexpr int N = LEN;
+  static constexpr int r0 = LEN <= 32 ? 4 : LEN == 96 ? 8 : LEN == 192 ? 12 : 6;
+  static constexpr int r1 = LEN == 384 ? 8 : LEN / r0;
+  static constexpr int passes = LEN == 384 ? 3 : 2;
+  static constexpr int T = LEN / (r0 < r1 ? r0 : r1);
+  static constexpr int radix(int s) { return s == 0 ? r0 : s == 1 ? r1 : LEN / (r0 * r1); }
+  static constexpr int ns(int s) { return s == 0 ? 1 : s == 1 ? r0 : r0 * r1; }
+};
+template <int N>
+struct has_split : std::integral_constant<bool, N == 16 || N == 24 || N == 32 || N == 48 || N == 96 || N == 192 ||
+                                                    N == 384> {};
+// The plan of a length's own kernels (the persistent batch and the bulk-copy
+// schedules keep RegPlan's thread counts).
+template <int N>
+using plan_for = typename std::conditional<has_split<N>::value, SplitPlan<N>, RegPlan<N>>::type;
+// Threads of a CTA at most: 256, or 512 where a line takes 64.
+template <class RP>
+constexpr int max_threads() { return RP::T > 32 ? 512 : 256; }
+
 // LD_SHARED: ld reads the shared buffer (the first pass then waits for all
 // reads before writing); later passes always read all before their stores.
-template <typename T, bool INV, int N, int S, int TWS, bool LD_SHARED, int PAD, class Ld, class St>
+template <typename T, bool INV, class RP, int S, int TWS, bool LD_SHARED, int PAD, class Ld, class St>
 __device__ __forceinline__ void pass(Ld& ld, St& st, cpx<T>* ln, int es, int t0, const cpx<T>* __restrict__ tw) {
-  using namespace ctfft;
-  constexpr int NST = nst(N, 16);
-  constexpr int R = radix_at(N, S, 16);
-  constexpr int NS = ns_at(N, S, 16);
-  constexpr int NB = N / R;
-  constexpr int TPL = N / 16;
-  constexpr int IT = NB / TPL;
+  constexpr int N = RP::N, NST = RP::passes, R = RP::radix(S), NS = RP::ns(S);
+  constexpr int NB = N / R, TPL = RP::T, IT = (NB + TPL - 1) / TPL;
   constexpr int TSTEP = N / (NS * R);
-  static_assert(IT * R == 16, "a thread holds 16 elements per pass");
   cpx<T> v[IT][R];
 #pragma unroll
   for (int it = 0; it < IT; ++it) {
     const int t = t0 + it * TPL;
+    if (NB % TPL != 0 && t >= NB) continue;
 #pragma unroll
     for (int q = 0; q < R; ++q) {
       const int e = t + q * NB;
@@ -429,6 +520,7 @@ __device__ __forceinline__ void pass(Ld& ld, St& st, cpx<T>* ln, int es, int t0,
 #pragma unroll
   for (int it = 0; it < IT; ++it) {
     const int t = t0 + it * TPL;
+    if (NB % TPL != 0 && t >= NB) continue;
     const int q0 = t / NS, k = t - q0 * NS;
     if (NS > 1) {
       const int e1 = TSTEP * TWS * k;
@@ -450,26 +542,31 @@ __device__ __forceinline__ void pass(Ld& ld, St& st, cpx<T>* ln, int es, int t0,
   if (S + 1 < NST) __syncthreads();
 }
 
-template <typename T, bool INV, int N, int S, int TWS, bool LD_SHARED, int PAD, class Ld, class St>
+template <typename T, bool INV, class RP, int S, int TWS, bool LD_SHARED, int PAD, class Ld, class St>
 __device__ __forceinline__ void run_from(Ld& ld, St& st, cpx<T>* ln, int es, int t0, const cpx<T>* __restrict__ tw) {
-  if constexpr (S < ctfft::nst(N, 16)) {
-    pass<T, INV, N, S, TWS, LD_SHARED, PAD>(ld, st, ln, es, t0, tw);
-    run_from<T, INV, N, S + 1, TWS, LD_SHARED, PAD>(ld, st, ln, es, t0, tw);
+  if constexpr (S < RP::passes) {
+    pass<T, INV, RP, S, TWS, LD_SHARED, PAD>(ld, st, ln, es, t0, tw);
+    run_from<T, INV, RP, S + 1, TWS, LD_SHARED, PAD>(ld, st, ln, es, t0, tw);
   }
 }
 
-// Transform of the CTA's lines (N/16 threads per line, every thread of the
-// CTA calls; t0 in [0, N/16) is the thread's rank within its line).  `tw`
-// holds exp(-2 pi i t/(N*TWS)) and must be visible to all threads before the
-// second pass (the barrier after the first pass suffices when it is written
-// before the call).  The caller synchronises after the call before reusing
-// the buffer.
+// Transform of the CTA's lines by plan RP (RP::T threads per line, every
+// thread of the CTA calls; t0 in [0, RP::T) is the thread's rank within its
+// line).  `tw` holds exp(-2 pi i t/(N*TWS)) and must be visible to all threads
+// before the second pass (the barrier after the first pass suffices when it is
+// written before the call).  The caller synchronises after the call before
+// reusing the buffer.
+template <typename T, bool INV, class RP, int TWS, bool LD_SHARED, int PAD = PAD_ROWS, class Ld, class St>
+__device__ __forceinline__ void run_plan(Ld&& ld, St&& st, cpx<T>* ln, int es, int t0, const cpx<T>* __restrict__ tw) {
+  run_from<T, INV, RP, 0, TWS, LD_SHARED, PAD>(ld, st, ln, es, t0, tw);
+}
 template <typename T, bool INV, int N, int TWS, bool LD_SHARED, int PAD = PAD_ROWS, class Ld, class St>
 __device__ __forceinline__ void run(Ld&& ld, St&& st, cpx<T>* ln, int es, int t0, const cpx<T>* __restrict__ tw) {
   static_assert((N & (N - 1)) == 0 && N >= 16 && N <= 512, "power-of-two length");
-  run_from<T, INV, N, 0, TWS, LD_SHARED, PAD>(ld, st, ln, es, t0, tw);
+  run_from<T, INV, RegPlan<N>, 0, TWS, LD_SHARED, PAD>(ld, st, ln, es, t0, tw);
 }
 
+// lengths with a RegPlan
 template <int N> struct is_rg : std::integral_constant<bool, (N >= 16 && N <= 512 && (N & (N - 1)) == 0)> {};
 
 }  // namespace rgfft

@@ -63,22 +63,22 @@ bool batch_dims_ok(int nx, int ny, int nz) { return len_ok(nx) && len_ok(ny) && 
 
 // x passes of a radix-3 nx/2: as many lines as keep the tile within 4096 reals
 // (at most 64), as the graph form's default
-int batch_lpb(int nx) {
+constexpr int batch_lpb(int nx) {
   int l = 1;
   while (2 * l <= 4096 / nx && 2 * l <= 64) l *= 2;
   return l;
 }
 // z (16) and y (8) columns of a radix-3 length, fewer when the tile would not fit
-int batch_tkx(int n, bool zpass) {
+constexpr int batch_tkx(int n, bool zpass) {
   int t = zpass ? 16 : 8;
   while (t > 2 && 8 * (2 * (size_t)t * n + n) > 160 * 1024) t /= 2;
   return t;
 }
 
 namespace {
-// tiles of a transform pass along a length-n direction: power-of-two lengths
-// run the register-staged form with 4096 / n lines (256 threads); radix-3
-// lengths the shared-memory form with `cols` lines
+// tiles of a transform pass along a length-n direction: 4096 / n lines for
+// power-of-two lengths, `cols` lines for radix-3 ones (256 threads share them:
+// BatchPlan)
 unsigned lines_per_tile(int n, int cols) { return pow2(n) ? 4096u / (unsigned)n : (unsigned)cols; }
 constexpr size_t kRhoCellsPerTile = 65536;     // rho_0 reduction: 256 threads x 256 cells
 constexpr size_t kFacesPerThreadCC = 16;        // correction check: v faces per thread
@@ -135,11 +135,9 @@ size_t batch_smem(int nx, int ny, int nz) {
   const size_t tj = (size_t)(kRhsThreads / nx) * kBatchRhsLines;
   size_t m = sizeof(df) * (size_t)nx * (2 * (tj + 2) + tj) +
              (rhs_slots_in_smem(kBatchRhsLines) ? sizeof(double) * rhs_slots(kBatchRhsLines, 2) * kRhsThreads : 0);
-  const int lx = (int)lines_per_tile(nx / 2, batch_lpb(nx));
-  m = std::max(m, pow2(nx / 2) ? xrg_smem(nx, lx) : xfwd_smem<float>(nx, lx));
-  m = std::max(m, pow2(nx / 2) ? xrg_smem(nx, lx) : xinv_smem<float>(nx, lx));
-  m = std::max(m, pow2(nz) ? rg_smem<float>(nz, 4096 / nz) : zfft_smem<float>(nz, batch_tkx(nz, true)));
-  m = std::max(m, pow2(ny) ? rg_smem<float>(ny, 4096 / ny) : zfft_smem<float>(ny, batch_tkx(ny, false)));
+  m = std::max(m, xrg_smem(nx, (int)lines_per_tile(nx / 2, batch_lpb(nx))));
+  m = std::max(m, rg_smem<float>(nz, (int)lines_per_tile(nz, batch_tkx(nz, true))));
+  m = std::max(m, rg_smem<float>(ny, (int)lines_per_tile(ny, batch_tkx(ny, false))));
   return m;
 }
 
@@ -246,20 +244,29 @@ __device__ __forceinline__ void on_len(int n, F&& f) {
   }
 }
 
+// The radices of a length's own kernels (plan_for, so the same bits) on the
+// 256 / L threads that each of a tile's L lines has here.
+template <int LEN, int L>
+struct BatchPlan {
+  using Own = rgfft::plan_for<LEN>;
+  static constexpr int N = LEN, T = kBatchThreads / L, passes = Own::passes;
+  static constexpr int radix(int s) { return Own::radix(s); }
+  static constexpr int ns(int s) { return Own::ns(s); }
+};
+constexpr bool is_pow2(int n) { return (n & (n - 1)) == 0; }
+constexpr int x_lines_of(int m) { return is_pow2(m) ? 4096 / m : batch_lpb(2 * m); }
+constexpr int z_cols_of(int n) { return is_pow2(n) ? 4096 / n : batch_tkx(n, true); }
+constexpr int y_cols_of(int n) { return is_pow2(n) ? 4096 / n : batch_tkx(n, false); }
+
 // forward x pass of f (SRC_FDF) or of the residual (SRC_RESID), tile t of nt
 template <int SRC>
 __device__ __noinline__ void x_forward(const BatchGrid* __restrict__ Bp, uint32_t t, uint32_t nt) {
   const BatchGrid& B = *Bp;
   on_xhalf(B.g.nx / 2, [&](auto MC) {
     constexpr int M = decltype(MC)::value;
-    if constexpr (rgfft::is_rg<M>::value) {
-      xfwd_rg_body<SRC, M, false, false>(B.g, B.in, B.sc, SRC == SRC_RESID ? -1 : 0, B.fdf, B.pdf, B.spec, B.tw_x,
-                                         4096 / M, t, nt);
-    } else {
-      RadixPlan rp;  // (compile-time lengths: the radix plan is not read)
-      xfwd_body<float, SRC, true, M, false>(B.g, B.in, B.sc, SRC == SRC_RESID ? -1 : 0, B.fdf, B.pdf, B.spec, rp,
-                                            B.tw_x, B.lpb, t, nt);
-    }
+    constexpr int L = x_lines_of(M);
+    xfwd_rg_body<SRC, M, false, false, BatchPlan<M, L>>(B.g, B.in, B.sc, SRC == SRC_RESID ? -1 : 0, B.fdf, B.pdf, B.spec,
+                                                        B.tw_x, L, t, nt);
   });
 }
 
@@ -270,12 +277,8 @@ __device__ __noinline__ void x_inverse(const BatchGrid* __restrict__ Bp, uint32_
   const BatchGrid& B = *Bp;
   on_xhalf(B.g.nx / 2, [&](auto MC) {
     constexpr int M = decltype(MC)::value;
-    if constexpr (rgfft::is_rg<M>::value) {
-      xinv_rg_body<MODE, M, false>(B.g, B.spec, nullptr, B.pdf, B.scale, B.tw_x, 4096 / M, nullptr, B.sc, t, nt);
-    } else {
-      RadixPlan rp;  // (compile-time lengths: the radix plan is not read)
-      xinv_body<float, MODE, M>(B.g, B.spec, nullptr, B.pdf, B.scale, rp, B.tw_x, B.lpb, nullptr, B.sc, t, nt);
-    }
+    constexpr int L = x_lines_of(M);
+    xinv_rg_body<MODE, M, false, BatchPlan<M, L>>(B.g, B.spec, nullptr, B.pdf, B.scale, B.tw_x, L, nullptr, B.sc, t, nt);
   });
 }
 
@@ -286,12 +289,8 @@ __device__ __noinline__ void z_pass(const BatchGrid* __restrict__ Bp, uint32_t t
   DevScalars* fin = INV ? nullptr : B.sc;
   on_len(B.g.nz, [&](auto NC) {
     constexpr int N = decltype(NC)::value;
-    if constexpr (rgfft::is_rg<N>::value) {
-      zfft_rg_body<float, INV, N>(B.g, B.spec, B.tw_z, 4096 / N, nullptr, fin, t, nt);
-    } else {
-      RadixPlan rp;  // (compile-time lengths: the radix plan is not read)
-      zfft_body<float, INV, N>(B.g, B.spec, rp, B.tw_z, B.tkx, nullptr, fin, t, nt);
-    }
+    constexpr int L = z_cols_of(N);
+    zfft_rg_body<float, INV, N, BatchPlan<N, L>>(B.g, B.spec, B.tw_z, L, nullptr, fin, t, nt);
   });
 }
 
@@ -302,11 +301,9 @@ __device__ __noinline__ void y_pass(const BatchGrid* __restrict__ Bp, uint32_t t
     constexpr int N = decltype(NC)::value;
     if constexpr (N == 256) {  // the radix-16 x 16 form with the divide in registers, as the graph form
       ydct256_body(B.g, B.spec, B.tw_y, B.wq_y, B.lam_x, B.lam_y, B.lam_z, 16, B.sc, t, nt);
-    } else if constexpr (rgfft::is_rg<N>::value) {
-      ydct_rg_body<float, N>(B.g, B.spec, B.tw_y, B.wq_y, B.lam_x, B.lam_y, B.lam_z, 4096 / N, B.sc, t, nt);
     } else {
-      RadixPlan rp;  // (compile-time lengths: the radix plan is not read)
-      ydct_body<float, N>(B.g, B.spec, rp, B.tw_y, B.wq_y, B.lam_x, B.lam_y, B.lam_z, B.tky, B.sc, t, nt);
+      constexpr int L = y_cols_of(N);
+      ydct_rg_body<float, N, BatchPlan<N, L>>(B.g, B.spec, B.tw_y, B.wq_y, B.lam_x, B.lam_y, B.lam_z, L, B.sc, t, nt);
     }
   });
 }

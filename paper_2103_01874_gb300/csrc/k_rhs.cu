@@ -295,7 +295,10 @@ __global__ void __launch_bounds__(kRhsThreads, CPT == 4 ? 2 : 1)
   }
 }
 
-__global__ void k_finish_sums(GridDev g, DevScalars* sc) { finish_sums(sc, g); }
+__global__ void k_finish_sums(GridDev g, DevScalars* sc) {
+  pdl_enter();
+  finish_sums(sc, g);
+}
 
 // Column-stack form of the march (rhs.cuh): one CTA of BT threads at most per
 // tile.  What bounds it: instruction issue and the latency of a step's loads
@@ -467,7 +470,7 @@ cudaError_t raise_smem(K kernel, size_t* dyn_max) {
 }  // namespace
 
 cudaError_t launch_finish_sums(const GridDev& g, DevScalars* sc, cudaStream_t st) {
-  k_finish_sums<<<1, 256, 0, st>>>(g, sc);
+  launch_pdl(k_finish_sums, 1, 256, 0, st, g, sc);
   return cudaGetLastError();
 }
 

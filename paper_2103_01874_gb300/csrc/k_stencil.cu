@@ -28,6 +28,7 @@ __global__ void __launch_bounds__(256) k_correct_pre(GridDev g, double dt, const
                                                      const df* __restrict__ vpre, const df* __restrict__ wpre,
                                                      const df* __restrict__ pdf, double* p64, const DevScalars* sc,
                                                      double* u_out, double* v_out, double* w_out) {
+  pdl_enter();
   const uint32_t nx = (uint32_t)g.nx, ny = (uint32_t)g.ny;
   const uint32_t total = (uint32_t)g.nz * (ny + 1) * nx;
   const StencilConst K = sc->K;
@@ -90,6 +91,7 @@ __global__ void __launch_bounds__(256) k_correct_pre(GridDev g, double dt, const
 // every thread reads u*, v*, w* only at the faces it writes.
 __global__ void __launch_bounds__(256) k_correct_full(GridDev g, StencilIn in, const DevScalars* sc, double* u_out,
                                                       double* v_out, double* w_out) {
+  pdl_enter();
   const size_t nx = (size_t)g.nx, ny = (size_t)g.ny;
   const size_t total = (size_t)g.nz * (ny + 1) * nx;
   const StencilConst K = sc->K;
@@ -128,6 +130,7 @@ __global__ void __launch_bounds__(256) k_correct_full(GridDev g, StencilIn in, c
 }
 
 __global__ void __launch_bounds__(256) k_df_to_d(const df* __restrict__ a, double* out, size_t n) {
+  pdl_enter();
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
     out[i] = df2d(a[i]);
 }
@@ -154,6 +157,7 @@ __global__ void k_make_const(GridDev g, DevScalars* sc, double dt) {
 }
 
 __global__ void k_set_rho0(DevScalars* sc, double rho0) {
+  pdl_enter();
   if (threadIdx.x == 0) sc->rho0_bits = (unsigned long long)__double_as_longlong(rho0);
 }
 
@@ -169,6 +173,7 @@ __global__ void __launch_bounds__(256) k_div_constraint(size_t n, const double* 
                                                         const double* __restrict__ rho_l,
                                                         const unsigned char* __restrict__ mask, double* S,
                                                         double* rho) {
+  pdl_enter();
   const df one = {1.0f, 0.0f};
   for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < n; c += (size_t)gridDim.x * blockDim.x) {
     const double cd = __ldg(C + c);
@@ -215,8 +220,8 @@ size_t one_wave() {
 cudaError_t launch_div_constraint(size_t n, const double* C, const double* comp_g, const double* comp_l,
                                   const double* mdot, const double* rho_g, const double* rho_l,
                                   const unsigned char* mask, double* S, double* rho, cudaStream_t st) {
-  k_div_constraint<<<grid_for(n, (size_t)152 * 16), 256, 0, st>>>(n, C, comp_g, comp_l, mdot, rho_g, rho_l, mask, S,
-                                                                  rho);
+  launch_pdl(k_div_constraint, grid_for(n, (size_t)152 * 16), 256, 0, st, n, C, comp_g, comp_l, mdot, rho_g, rho_l, mask,
+             S, rho);
   return cudaGetLastError();
 }
 
@@ -227,7 +232,7 @@ cudaError_t launch_init_scalars(DevScalars* sc, double rho0, double tol, int kee
 }
 
 cudaError_t launch_set_rho0(DevScalars* sc, double rho0, cudaStream_t st) {
-  k_set_rho0<<<1, 32, 0, st>>>(sc, rho0);
+  launch_pdl(k_set_rho0, 1, 32, 0, st, sc, rho0);
   return cudaGetLastError();
 }
 
@@ -245,15 +250,15 @@ cudaError_t launch_correct_pre(const GridDev& g, double dt, const df* upre, cons
                                const df* pdf, double* p64, const DevScalars* sc, double* u_out, double* v_out,
                                double* w_out, cudaStream_t st) {
   const size_t total = (size_t)g.nz * (g.ny + 1) * g.nx;
-  k_correct_pre<<<grid_for(total, one_wave<k_correct_pre>()), 256, 0, st>>>(g, dt, upre, vpre, wpre, pdf, p64, sc, u_out,
-                                                                   v_out, w_out);
+  launch_pdl(k_correct_pre, grid_for(total, one_wave<k_correct_pre>()), 256, 0, st, g, dt, upre, vpre, wpre, pdf, p64, sc,
+             u_out, v_out, w_out);
   return cudaGetLastError();
 }
 
 cudaError_t launch_correct_full(const GridDev& g, const StencilIn& in, const DevScalars* sc, double* u_out,
                                 double* v_out, double* w_out, cudaStream_t st) {
   const size_t total = (size_t)g.nz * (g.ny + 1) * g.nx;
-  k_correct_full<<<grid_for(total, one_wave<k_correct_full>()), 256, 0, st>>>(g, in, sc, u_out, v_out, w_out);
+  launch_pdl(k_correct_full, grid_for(total, one_wave<k_correct_full>()), 256, 0, st, g, in, sc, u_out, v_out, w_out);
   return cudaGetLastError();
 }
 
@@ -265,7 +270,7 @@ cudaError_t launch_correct_check(const GridDev& g, const df* upre, const df* vpr
 }
 
 cudaError_t launch_df_to_d(const df* a, double* out, size_t n, cudaStream_t st) {
-  k_df_to_d<<<grid_for(n, (size_t)152 * 32), 256, 0, st>>>(a, out, n);
+  launch_pdl(k_df_to_d, grid_for(n, (size_t)152 * 32), 256, 0, st, a, out, n);
   return cudaGetLastError();
 }
 

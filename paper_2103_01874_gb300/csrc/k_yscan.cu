@@ -1,4 +1,5 @@
 // y pass of the FP32 solve with walls as a tridiagonal solve in scan form.
+#include "pdl.cuh"
 #include "ppe_internal.h"
 
 namespace ppe {
@@ -104,6 +105,7 @@ __global__ void __launch_bounds__(256, (S <= 4 ? 4 : (S == 8 ? 3 : (S == 16 ? 2 
                                                       const int* __restrict__ line_off,
                                                       const int* __restrict__ line_len, float a,
                                                       const DevScalars* zsc) {
+  pdl_enter();
   constexpr int L = 16, T = 16;
   __shared__ float sA[T][L];
   __shared__ cpx<float> sB[T][L];
@@ -233,12 +235,12 @@ cudaError_t launch_ythomas_scan(const GridDev& g, cpx<float>* spec, const float*
   const int nxh = g.nx / 2 + 1;
   const int grid = g.nz * ((nxh + 15) / 16);
   switch (yscan_elems(g.ny)) {
-    case 1: k_ythomas_scan<1><<<grid, 256, 0, st>>>(g, spec, tab, line_off, line_len, a, zsc); break;
-    case 2: k_ythomas_scan<2><<<grid, 256, 0, st>>>(g, spec, tab, line_off, line_len, a, zsc); break;
-    case 4: k_ythomas_scan<4><<<grid, 256, 0, st>>>(g, spec, tab, line_off, line_len, a, zsc); break;
-    case 8: k_ythomas_scan<8><<<grid, 256, 0, st>>>(g, spec, tab, line_off, line_len, a, zsc); break;
-    case 16: k_ythomas_scan<16><<<grid, 256, 0, st>>>(g, spec, tab, line_off, line_len, a, zsc); break;
-    case 32: k_ythomas_scan<32><<<grid, 256, 0, st>>>(g, spec, tab, line_off, line_len, a, zsc); break;
+    case 1: launch_pdl(k_ythomas_scan<1>, grid, 256, 0, st, g, spec, tab, line_off, line_len, a, zsc); break;
+    case 2: launch_pdl(k_ythomas_scan<2>, grid, 256, 0, st, g, spec, tab, line_off, line_len, a, zsc); break;
+    case 4: launch_pdl(k_ythomas_scan<4>, grid, 256, 0, st, g, spec, tab, line_off, line_len, a, zsc); break;
+    case 8: launch_pdl(k_ythomas_scan<8>, grid, 256, 0, st, g, spec, tab, line_off, line_len, a, zsc); break;
+    case 16: launch_pdl(k_ythomas_scan<16>, grid, 256, 0, st, g, spec, tab, line_off, line_len, a, zsc); break;
+    case 32: launch_pdl(k_ythomas_scan<32>, grid, 256, 0, st, g, spec, tab, line_off, line_len, a, zsc); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();

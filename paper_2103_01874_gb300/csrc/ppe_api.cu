@@ -1345,9 +1345,6 @@ ppe_status batch_persistent(ppe_batch_t B, int n, const ppe_plan_t* plans, const
     G.tol = P->opt.refine_tol;
     G.scale = 1.0 / ((double)(P->g.nx / 2) * (double)P->g.nz);
     G.smax = P->opt.max_sweeps;
-    G.lpb = batch_lpb(P->g.nx);
-    G.tkx = batch_tkx(P->g.nz, true);
-    G.tky = batch_tkx(P->g.ny, false);
     G.kc = P->g.nz < 8 ? P->g.nz : 8;
     G.stage0 = kBatchStages * i;
   }

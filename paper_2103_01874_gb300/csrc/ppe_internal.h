@@ -248,7 +248,7 @@ struct BatchGrid {            // one grid of the batch (device copy, read-only i
   double *out_p, *out_u, *out_v, *out_w;
   double rho0, tol, scale;    // rho0 <= 0: min(rho); scale 1 / ((nx/2) nz)
   int smax;                   // refinement sweeps at most (>= 1)
-  int lpb, tkx, tky, kc;      // tiles of the x passes (radix-3 nx), z and y passes (radix-3), RHS chunk
+  int kc;                     // RHS chunk
   int stage0;                 // the grid's first stage counter (kBatchStages per grid)
 };
 struct BatchItem {            // tiles tile0 .. tile0 + count - 1 of one stage of one grid
@@ -270,8 +270,6 @@ unsigned batch_stage_tiles(int nx, int ny, int nz, bool rho_given, int stage);
 // tiles per queue item of a stage: about `grain` elements (cells, faces or
 // spectrum values) per item, at most 255 tiles
 unsigned batch_stage_chunk(int nx, int ny, int nz, int stage, long grain);
-int batch_lpb(int nx);                                   // x-pass lines per tile (radix-3 nx/2)
-int batch_tkx(int n, bool zpass);                        // z / y columns per tile (radix-3 lengths)
 size_t batch_smem(int nx, int ny, int nz);               // dynamic shared memory of the grid's largest stage
 // queue of stages [first, kBatchStages) of every grid: grids in windows of
 // `window`, stage-major within a window, window w offset by w * stagger stages

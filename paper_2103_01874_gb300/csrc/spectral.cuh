@@ -41,6 +41,9 @@ __device__ __forceinline__ int ilog2_dev(int v) { return __ffs(v) - 1; }
 
 // FP32 and pair passes have compile-time-length instances (register-staged
 // for powers of two); FP64 passes run on run-time radix plans
+// lengths with a register-staged FP32 pass
+template <int N>
+struct has_rg : std::integral_constant<bool, rgfft::is_rg<N>::value || rgfft::has_split<N>::value> {};
 template <typename T>
 struct has_ct_lengths : std::integral_constant<bool, sizeof(T) == 4 || std::is_same<T, dd>::value> {};
 
@@ -252,6 +255,7 @@ template <typename T, int SRC, bool DO_FFT, int N, bool OPEN = false>
 __global__ void __launch_bounds__(256) k_xfwd(GridDev g, StencilIn in, DevScalars* sc, int slot, df* fdf,
                                               const df* __restrict__ pdf, cpx<T>* spec, RadixPlan rp,
                                               const cpx<T>* __restrict__ tw, int lpb) {
+  pdl_enter();
   xfwd_body<T, SRC, DO_FFT, N, OPEN>(g, in, sc, slot, fdf, pdf, spec, rp, tw, lpb, blockIdx.x, gridDim.x);
 }
 
@@ -276,24 +280,24 @@ struct PlaneLanes {
 };
 __device__ __forceinline__ PlaneLanes plane_lanes(int L) { return {L < 8 ? L : 8, 32 / (L < 8 ? L : 8)}; }
 
-// Register-staged forward x pass (FP32, nx = 2M, M a power of two; rgfft in
-// fft.cuh).  A CTA of L * M/16 threads owns L consecutive x-lines; thread
+// Register-staged forward x pass (FP32, nx = 2M, M a length with a plan; rgfft
+// in fft.cuh).  A CTA of L * RP::T threads owns L consecutive x-lines; thread
 // (line, t) forms the packed values z_e = x_{2e} + i x_{2e+1} of its first
-// FFT pass (e = t + q M/16) straight from the source -- f (FP64), f as pairs,
+// FFT pass (e = t + q M/R) straight from the source -- f (FP64), f as pairs,
 // or the residual f - L p in pair arithmetic, two cells per 16-byte load --
 // the last pass leaves Z in shared memory and the untangle writes the nx/2 + 1
 // half spectrum.  Same cell arithmetic as k_xfwd.
 // PL: the spectrum in the plane layout [kx][line] (GridDev::spec_planes).
-template <int SRC, int M, bool OPEN, bool PL = false>
+template <int SRC, int M, bool OPEN, bool PL = false, class RP = rgfft::RegPlan<M>>
 __device__ __forceinline__ void xfwd_rg_body(GridDev g, StencilIn in, DevScalars* sc, int slot, df* fdf,
                                                  const df* pdf, cpx<float>* spec,
                                                  const cpx<float>* tw, int L, uint32_t bid, uint32_t nblk) {
   using T = float;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (SRC == SRC_RESID && slot < 0) slot = sc->iter;  // residual slot chosen on the device
-  constexpr int TPL = M / 16, nx = 2 * M, nxh = M + 1, LS = xstride<PL>(M);
+  constexpr int TPL = RP::T, nx = 2 * M, nxh = M + 1, LS = xstride<PL>(M);
   const uint32_t nlines = (uint32_t)g.ny * (uint32_t)g.nz;
-  const int ll = (int)threadIdx.x / TPL, t0 = (int)threadIdx.x & (TPL - 1);
+  const int ll = (int)threadIdx.x / TPL, t0 = (int)threadIdx.x % TPL;
   const uint32_t l0 = bid * (uint32_t)L;
   const uint32_t line = l0 + ll;
   const bool valid = line < nlines;
@@ -307,10 +311,9 @@ __device__ __forceinline__ void xfwd_rg_body(GridDev g, StencilIn in, DevScalars
   if constexpr (SRC == SRC_F) {
     const double2* fl = reinterpret_cast<const double2*>(in.f + c0);
     float4* fo = fdf ? reinterpret_cast<float4*>(fdf + c0) : nullptr;
-    // a caller's f off a 16-byte boundary is read with 8-byte loads (the plane
-    // layout has no other forward pass to fall back to)
-    const bool f16 = !PL || ((uintptr_t)in.f & 15u) == 0;
-    rgfft::run<T, false, M, 2, false>(
+    // a caller's f off a 16-byte boundary is read with 8-byte loads
+    const bool f16 = ((uintptr_t)in.f & 15u) == 0;
+    rgfft::run_plan<T, false, RP, 2, false>(
         [&](int e) -> cpx<T> {
           if (!valid) return {(T)0, (T)0};
           const double2 x = f16 ? __ldg(fl + e) : make_double2(__ldg(in.f + c0 + 2 * e), __ldg(in.f + c0 + 2 * e + 1));
@@ -324,7 +327,7 @@ __device__ __forceinline__ void xfwd_rg_body(GridDev g, StencilIn in, DevScalars
   } else if constexpr (SRC == SRC_FDF) {
     // f as pairs, written by the right-hand-side kernel (which also took ||f||)
     const float4* fl = reinterpret_cast<const float4*>(fdf + c0);
-    rgfft::run<T, false, M, 2, false>(
+    rgfft::run_plan<T, false, RP, 2, false>(
         [&](int e) -> cpx<T> {
           if (!valid) return {(T)0, (T)0};
           const float4 q = fl[e];
@@ -411,11 +414,11 @@ __device__ __forceinline__ void xfwd_rg_body(GridDev g, StencilIn in, DevScalars
       return {r0, r1};
     };
     if (p0f)
-      rgfft::run<T, false, M, 2, false>(
+      rgfft::run_plan<T, false, RP, 2, false>(
           [&](int e) -> cpx<T> { return valid ? cell2(e, std::true_type{}) : cpx<T>{(T)0, (T)0}; }, put,
           buf + ll * LS, 1, t0, tws);
     else
-      rgfft::run<T, false, M, 2, false>(
+      rgfft::run_plan<T, false, RP, 2, false>(
           [&](int e) -> cpx<T> { return valid ? cell2(e, std::false_type{}) : cpx<T>{(T)0, (T)0}; }, put,
           buf + ll * LS, 1, t0, tws);
   }
@@ -459,11 +462,11 @@ __device__ __forceinline__ void xfwd_rg_body(GridDev g, StencilIn in, DevScalars
   }
 }
 template <int SRC, int M, bool OPEN, bool PL = false>
-__global__ void __launch_bounds__(256) k_xfwd_rg(GridDev g, StencilIn in, DevScalars* sc, int slot, df* fdf,
+__global__ void __launch_bounds__(rgfft::max_threads<rgfft::plan_for<M>>()) k_xfwd_rg(GridDev g, StencilIn in, DevScalars* sc, int slot, df* fdf,
                                                  const df* __restrict__ pdf, cpx<float>* spec,
                                                  const cpx<float>* __restrict__ tw, int L) {
   pdl_enter();
-  xfwd_rg_body<SRC, M, OPEN, PL>(g, in, sc, slot, fdf, pdf, spec, tw, L, blockIdx.x, gridDim.x);
+  xfwd_rg_body<SRC, M, OPEN, PL, rgfft::plan_for<M>>(g, in, sc, slot, fdf, pdf, spec, tw, L, blockIdx.x, gridDim.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -504,14 +507,16 @@ __device__ __forceinline__ void zfft_body(GridDev g, cpx<T>* spec, RadixPlan rp,
 template <typename T, bool INV, int N>
 __global__ void __launch_bounds__(256) k_zfft(GridDev g, cpx<T>* spec, RadixPlan rp, const cpx<T>* __restrict__ tw,
                                               int tkx, const DevScalars* sc, DevScalars* fin) {
+  pdl_enter();
   zfft_body<T, INV, N>(g, spec, rp, tw, tkx, sc, fin, blockIdx.x, gridDim.x);
 }
 
-// Register-staged z pass (FP32, power-of-two nz; rgfft in fft.cuh): one CTA
-// per (j, tile of L kx columns), L * nz/16 threads; the first pass reads the
+// Register-staged z pass (FP32, nz a length with a plan, and pairs, nz a power
+// of two; rgfft in fft.cuh): one CTA per (j, tile of L kx columns), L * RP::T
+// threads; the first pass reads the
 // columns from the spectrum and the last pass writes them back, so each
 // element crosses shared memory once.
-template <typename T, bool INV, int N>
+template <typename T, bool INV, int N, class RP = rgfft::RegPlan<N>>
 __device__ __forceinline__ void zfft_rg_body(GridDev g, cpx<T>* spec, const cpx<T>* tw, int L,
                                                  const DevScalars* sc, DevScalars* fin, uint32_t bid, uint32_t nblk) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -528,18 +533,21 @@ __device__ __forceinline__ void zfft_rg_body(GridDev g, cpx<T>* spec, const cpx<
   const bool valid = kx0 + line < nxh;
   const uint32_t rs = (uint32_t)g.ny * nxh;  // kz stride (32-bit offsets: spectra below 2^32 elements)
   cpx<T>* col = spec + (j * nxh + kx0 + line);
-  rgfft::run<T, INV, N, 1, false>(
+  rgfft::run_plan<T, INV, RP, 1, false>(
       [&](int e) { return valid ? col[(uint32_t)e * rs] : cpx<T>{(T)0, (T)0}; },
       [&](int e, cpx<T> v) {
         if (valid) col[(uint32_t)e * rs] = v;
       },
       buf + line, L, t0, tws);
 }
+// (pairs keep RegPlan: their split plans would not fit the registers)
+template <typename T, int N>
+using z_plan = typename std::conditional<sizeof(T) == 4, rgfft::plan_for<N>, rgfft::RegPlan<N>>::type;
 template <typename T, bool INV, int N>
-__global__ void __launch_bounds__(256) k_zfft_rg(GridDev g, cpx<T>* spec, const cpx<T>* __restrict__ tw, int L,
+__global__ void __launch_bounds__(rgfft::max_threads<z_plan<T, N>>()) k_zfft_rg(GridDev g, cpx<T>* spec, const cpx<T>* __restrict__ tw, int L,
                                                  const DevScalars* sc, DevScalars* fin) {
   pdl_enter();
-  zfft_rg_body<T, INV, N>(g, spec, tw, L, sc, fin, blockIdx.x, gridDim.x);
+  zfft_rg_body<T, INV, N, z_plan<T, N>>(g, spec, tw, L, sc, fin, blockIdx.x, gridDim.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -568,6 +576,7 @@ template <typename T>
 __global__ void __launch_bounds__(128) k_ythomas(GridDev g, cpx<T>* spec, const T* __restrict__ tab,
                                                  const int* __restrict__ line_off, const int* __restrict__ line_len,
                                                  T a, const DevScalars* sc) {
+  pdl_enter();
   if (sc && sc->done) return;
   const int nxh = g.nx / 2 + 1, ny = g.ny;
   const int kz = blockIdx.y;
@@ -745,15 +754,16 @@ __global__ void __launch_bounds__(256) k_ydct(GridDev g, cpx<T>* spec, RadixPlan
                                               const cpx<T>* __restrict__ wq, const T* __restrict__ lam_x,
                                               const T* __restrict__ lam_y, const T* __restrict__ lam_z, int tky,
                                               const DevScalars* zsc) {
+  pdl_enter();
   ydct_body<T, N>(g, spec, rp, tw, wq, lam_x, lam_y, lam_z, tky, zsc, blockIdx.x, gridDim.x);
 }
 
-// Register-staged form of k_ydct (FP32, power-of-two ny; rgfft in fft.cuh):
+// Register-staged form of k_ydct (FP32, ny a length with a plan; rgfft in fft.cuh):
 // the reordered line is read straight from the spectrum by the first pass of
 // the DCT-II's FFT, the eigenvalue division works on the shared buffer, and
 // the last pass of the inverse writes the reordered result back.  Same
 // arithmetic as k_ydct.
-template <typename T, int N>
+template <typename T, int N, class RP = rgfft::RegPlan<N>>
 __device__ __forceinline__ void ydct_rg_body(GridDev g, cpx<T>* spec, const cpx<T>* tw,
                                                  const cpx<T>* wq, const T* lam_x,
                                                  const T* lam_y, const T* lam_z, int L,
@@ -771,13 +781,15 @@ __device__ __forceinline__ void ydct_rg_body(GridDev g, cpx<T>* spec, const cpx<
   cpx<T>* col = spec + (kz * (uint32_t)N * nxh + kx0 + line);
   // v[p] = x_j with p = j/2 (even j) or N-1-(j-1)/2 (odd j)
   auto jof = [](int p) { return p < N / 2 ? 2 * p : 2 * (N - 1 - p) + 1; };
-  rgfft::run<T, false, N, 1, false>(
+  rgfft::run_plan<T, false, RP, 1, false>(
       [&](int p) { return valid ? col[(uint32_t)jof(p) * nxh] : cpx<T>{(T)0, (T)0}; },
       [&](int e, cpx<T> v) { buf[rgfft::row(e) * L + line] = v; }, buf + line, L, t0, tws);
   __syncthreads();
   const T inv_n = (T)1 / (T)N;
   const T lz = lam_z[kz];
   constexpr int npair = N / 2 + 1;
+  // 1/N times the reciprocal: with N a power of two that is the correctly
+  // rounded quotient; else one more rounding, the same in both of a pair's lines
 #pragma unroll 1
   for (int idx = threadIdx.x; idx < npair * L; idx += blockDim.x) {
     const int k = idx >> lg, c = idx & (L - 1);
@@ -788,8 +800,6 @@ __device__ __forceinline__ void ydct_rg_body(GridDev g, cpx<T>* spec, const cpx<
     if (k == 0) {
       const T lam = lxz + lam_y[0];
       const cpx<T> v0 = *Vk;
-      // inv_n / lam as inv_n * (1/lam): inv_n is a power of two, so the correctly
-      // rounded reciprocal times it is the correctly rounded quotient
       if (kx == 0 && kz == 0) {  // zero mode pinned (to the value that keeps p zero-mean)
         *Vk = {(T)zsc->zmode, (T)0};
         continue;
@@ -814,7 +824,7 @@ __device__ __forceinline__ void ydct_rg_body(GridDev g, cpx<T>* spec, const cpx<
     if (r != k) *Vr = cmul(wrc, cpx<T>{pr.x + pk.y, pr.y - pk.x});
   }
   __syncthreads();
-  rgfft::run<T, true, N, 1, true>(
+  rgfft::run_plan<T, true, RP, 1, true>(
       [&](int e) { return buf[rgfft::row(e) * L + line]; },
       [&](int e, cpx<T> v) { buf[rgfft::row(e) * L + line] = v; }, buf + line, L, t0, tws);
   __syncthreads();
@@ -826,12 +836,12 @@ __device__ __forceinline__ void ydct_rg_body(GridDev g, cpx<T>* spec, const cpx<
   }
 }
 template <typename T, int N>
-__global__ void __launch_bounds__(256, 4) k_ydct_rg(GridDev g, cpx<T>* spec, const cpx<T>* __restrict__ tw,
+__global__ void __launch_bounds__(rgfft::max_threads<rgfft::plan_for<N>>(), rgfft::plan_for<N>::T > 32 ? 2 : 4) k_ydct_rg(GridDev g, cpx<T>* spec, const cpx<T>* __restrict__ tw,
                                                  const cpx<T>* __restrict__ wq, const T* __restrict__ lam_x,
                                                  const T* __restrict__ lam_y, const T* __restrict__ lam_z, int L,
                                                  const DevScalars* zsc) {
   pdl_enter();
-  ydct_rg_body<T, N>(g, spec, tw, wq, lam_x, lam_y, lam_z, L, zsc, blockIdx.x, gridDim.x);
+  ydct_rg_body<T, N, rgfft::plan_for<N>>(g, spec, tw, wq, lam_x, lam_y, lam_z, L, zsc, blockIdx.x, gridDim.x);
 }
 
 // 256-point form of k_ydct_rg (radices 16 x 16) with the eigenvalue divide in
@@ -1028,10 +1038,11 @@ template <typename T, int MODE, int N>
 __global__ void __launch_bounds__(256) k_xinv(GridDev g, const cpx<T>* __restrict__ spec, double* p, df* pdf,
                                               double scale, RadixPlan rp, const cpx<T>* __restrict__ tw, int lpb,
                                               const DevScalars* sc, DevScalars* psc) {
+  pdl_enter();
   xinv_body<T, MODE, N>(g, spec, p, pdf, scale, rp, tw, lpb, sc, psc, blockIdx.x, gridDim.x);
 }
 
-// Register-staged inverse x pass (FP32, nx = 2M, M a power of two): thread
+// Register-staged inverse x pass (FP32, nx = 2M, M a length with a plan): thread
 // (line, t) forms the packed values Z_k of its first inverse-FFT pass from
 // X_k and X_{M-k} read straight from the spectrum, and the last pass stores
 // (or adds) the real pairs of cells 2n, 2n+1 with one 16-byte access.  Same
@@ -1039,7 +1050,7 @@ __global__ void __launch_bounds__(256) k_xinv(GridDev g, const cpx<T>* __restric
 // PL: the spectrum in the plane layout [kx][line]; the CTA's half spectra are
 // first copied (transposed) into the shared buffer, then the first pass reads
 // them there.
-template <int MODE, int M, bool PL = false>
+template <int MODE, int M, bool PL = false, class RP = rgfft::RegPlan<M>>
 __device__ __forceinline__ void xinv_rg_body(GridDev g, const cpx<float>* spec, double* p, df* pdf,
                                                  double scale, const cpx<float>* tw, int L,
                                                  const DevScalars* sc, DevScalars* psc, uint32_t bid, uint32_t nblk,
@@ -1047,9 +1058,9 @@ __device__ __forceinline__ void xinv_rg_body(GridDev g, const cpx<float>* spec, 
   using T = float;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (sc && sc->done) return;
-  constexpr int TPL = M / 16, nx = 2 * M, nxh = M + 1, LS = xstride<PL>(M);
+  constexpr int TPL = RP::T, nx = 2 * M, nxh = M + 1, LS = xstride<PL>(M);
   const uint32_t nlines = (uint32_t)g.ny * (uint32_t)g.nz;
-  const int ll = (int)threadIdx.x / TPL, t0 = (int)threadIdx.x & (TPL - 1);
+  const int ll = (int)threadIdx.x / TPL, t0 = (int)threadIdx.x % TPL;
   const uint32_t line = bid * (uint32_t)L + ll;
   const bool valid = line < nlines;
   cpx<T>* buf = reinterpret_cast<cpx<T>*>(smem_raw);
@@ -1124,12 +1135,12 @@ __device__ __forceinline__ void xinv_rg_body(GridDev g, const cpx<float>* spec, 
     }
   };
   if constexpr (MODE != XI_DF_ACC) {
-    rgfft::run<T, true, M, 2, PL, rgfft::PAD_ROWS>(ld, st, buf + ll * LS, 1, t0, tws);
+    rgfft::run_plan<T, true, RP, 2, PL>(ld, st, buf + ll * LS, 1, t0, tws);
   } else {
     // p += s x: the last pass leaves x in shared memory; the update then runs
     // over consecutive cell pairs with four read-modify-writes in flight
-    rgfft::run<T, true, M, 2, PL, rgfft::PAD_ROWS>(ld, [&](int e, cpx<T> v) { buf[ll * LS + rgfft::row(e)] = v; },
-                                  buf + ll * LS, 1, t0, tws);
+    rgfft::run_plan<T, true, RP, 2, PL>(ld, [&](int e, cpx<T> v) { buf[ll * LS + rgfft::row(e)] = v; }, buf + ll * LS,
+                                        1, t0, tws);
     __syncthreads();
     const uint32_t l0 = bid * (uint32_t)L;
     // the first sweep adds to the first solve's p in FP32 where it was kept so
@@ -1184,40 +1195,35 @@ __device__ __forceinline__ void xinv_rg_body(GridDev g, const cpx<float>* spec, 
   }
 }
 template <int MODE, int M, bool PL = false>
-__global__ void __launch_bounds__(256) k_xinv_rg(GridDev g, const cpx<float>* __restrict__ spec, double* p, df* pdf,
+__global__ void __launch_bounds__(rgfft::max_threads<rgfft::plan_for<M>>()) k_xinv_rg(GridDev g, const cpx<float>* __restrict__ spec, double* p, df* pdf,
                                                  double scale, const cpx<float>* __restrict__ tw, int L,
                                                  const DevScalars* sc, DevScalars* psc, float* p32) {
   pdl_enter();
-  xinv_rg_body<MODE, M, PL>(g, spec, p, pdf, scale, tw, L, sc, psc, blockIdx.x, gridDim.x, p32);
+  xinv_rg_body<MODE, M, PL, rgfft::plan_for<M>>(g, spec, p, pdf, scale, tw, L, sc, psc, blockIdx.x, gridDim.x, p32);
 }
 
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
-// Lines per CTA of the register-staged passes: the tuned tile, raised so that a
-// CTA (L * N/16 threads) holds at least one full warp and capped so that it
-// holds at most 256 threads (the kernels' launch bound).
+// Lines per CTA of the register-staged passes: the tuned tile (a power of two),
+// raised so that a CTA (L * RP::T threads) is a whole number of warps and
+// capped at the kernels' launch bound.
 // (nx/2) nz a power of two: the inverse transforms' scaling 1/((nx/2) nz) is exact in FP32
 inline bool is_pow2_scale(const GridDev& g) {
   const unsigned m = (unsigned)(g.nx / 2) * (unsigned)g.nz;
   return m != 0u && (m & (m - 1u)) == 0u;
 }
 
-template <int N>
+template <class RP>
 int rg_lines(int tile) {
-  constexpr int lo = 32 / (N / 16) > 1 ? 32 / (N / 16) : 1, hi = 256 / (N / 16);
+  int lo = 1, hi = 1;
+  while (lo * RP::T % 32 != 0) lo *= 2;
+  while (2 * hi * RP::T <= rgfft::max_threads<RP>()) hi *= 2;
   return tile < lo ? lo : (tile > hi ? hi : tile);
 }
 template <typename T>
 size_t rg_smem(int n, int L) {
   return sizeof(cpx<T>) * ((size_t)rgfft::rows(n) * L + (size_t)n);
-}
-// Lines per CTA of the register-staged x passes: the tuned x_lines, kept
-// within one warp .. 256 threads (M/16 threads per line).
-template <int M>
-int rg_xlines(int lpb) {
-  const int lo = 32 / (M / 16) > 1 ? 32 / (M / 16) : 1, hi = 256 / (M / 16);
-  return lpb < lo ? lo : (lpb > hi ? hi : lpb);
 }
 inline size_t xrg_smem(int nx, int L, bool pl = false) {
   return sizeof(cpx<float>) * ((size_t)(pl ? xrg_stride_pl(nx / 2) : xrg_stride(nx / 2)) * L + (size_t)nx);
@@ -1264,54 +1270,48 @@ cudaError_t launch_xfwd(int src, bool do_fft, const GridDev& g, const StencilIn&
   const int nlines = g.ny * g.nz;
   const int grid = (nlines + lpb - 1) / lpb;
   const size_t sm = xfwd_smem<T>(g.nx, lpb);
+  auto go_sm = [&](auto kernel) -> cudaError_t {  // the shared-memory form
+    cudaError_t e = allow_smem(kernel, sm);
+    if (e != cudaSuccess) return e;
+    launch_pdl(kernel, grid, 256, sm, st, g, in, sc, slot, fdf, pdf, spec, rp, tw, lpb);
+    return cudaGetLastError();
+  };
   return with_len<T>(g.nx / 2, [&](auto NC) -> cudaError_t {
     constexpr int N = decltype(NC)::value;
-    cudaError_t e;
-    if constexpr (sizeof(T) == 4 && rgfft::is_rg<N>::value) {
-      // (the register-staged form reads f with 16-byte loads)
-      // (the plane layout has only these instances: f must be 16-byte aligned)
-      if (do_fft && (src != SRC_F || ((uintptr_t)in.f & 15u) == 0 || g.spec_planes)) {
-        const int L = rg_xlines<N>(lpb);
-        const int gr = (nlines + L - 1) / L;
-        const size_t smr = xrg_smem(g.nx, L, g.spec_planes != 0);
-        auto go = [&](auto kernel) -> cudaError_t {
-          cudaError_t e2 = allow_smem(kernel, smr);
-          if (e2 != cudaSuccess) return e2;
-          launch_pdl(kernel, gr, L * (N / 16), smr, st, g, in, sc, slot, fdf, pdf, (cpx<float>*)spec, (const cpx<float>*)tw, L);
-          return cudaGetLastError();
-        };
+    if constexpr (sizeof(T) == 4 && has_rg<N>::value) {
+      if (!do_fft) return cudaErrorInvalidValue;
+      using RP = rgfft::plan_for<N>;
+      const int L = rg_lines<RP>(lpb);
+      const int gr = (nlines + L - 1) / L;
+      const size_t smr = xrg_smem(g.nx, L, g.spec_planes != 0);
+      auto go = [&](auto kernel) -> cudaError_t {
+        cudaError_t e2 = allow_smem(kernel, smr);
+        if (e2 != cudaSuccess) return e2;
+        launch_pdl(kernel, gr, L * RP::T, smr, st, g, in, sc, slot, fdf, pdf, (cpx<float>*)spec,
+                   (const cpx<float>*)tw, L);
+        return cudaGetLastError();
+      };
+      if constexpr (rgfft::is_rg<N>::value) {  // (the plane layout: powers of two)
         if (g.spec_planes) {
           if (src == SRC_F) return go(k_xfwd_rg<SRC_F, N, false, true>);
           if (src == SRC_FDF) return go(k_xfwd_rg<SRC_FDF, N, false, true>);
-          return go(k_xfwd_rg<SRC_RESID, N, false, true>);  // the plane layout has walls only
+          return go(k_xfwd_rg<SRC_RESID, N, false, true>);  // walls only
         }
-        if (src == SRC_F) return go(k_xfwd_rg<SRC_F, N, false>);
-        if (src == SRC_FDF) return go(k_xfwd_rg<SRC_FDF, N, false>);
-        if (!g.top_open) return go(k_xfwd_rg<SRC_RESID, N, false>);
-        return go(k_xfwd_rg<SRC_RESID, N, true>);
       }
-    }
-    if (g.spec_planes) return cudaErrorInvalidValue;  // plane layout: power-of-two nx/2 only
-    if (src == SRC_F) {
-      if ((e = allow_smem(k_xfwd<T, SRC_F, true, N>, sm)) != cudaSuccess) return e;
-      k_xfwd<T, SRC_F, true, N><<<grid, 256, sm, st>>>(g, in, sc, slot, fdf, pdf, spec, rp, tw, lpb);
-    } else if (src == SRC_FDF) {
-      if ((e = allow_smem(k_xfwd<T, SRC_FDF, true, N>, sm)) != cudaSuccess) return e;
-      k_xfwd<T, SRC_FDF, true, N><<<grid, 256, sm, st>>>(g, in, sc, slot, fdf, pdf, spec, rp, tw, lpb);
-    } else if (do_fft && !g.top_open) {
-      if ((e = allow_smem(k_xfwd<T, SRC_RESID, true, N>, sm)) != cudaSuccess) return e;
-      k_xfwd<T, SRC_RESID, true, N><<<grid, 256, sm, st>>>(g, in, sc, slot, fdf, pdf, spec, rp, tw, lpb);
-    } else if (do_fft) {
-      if ((e = allow_smem(k_xfwd<T, SRC_RESID, true, N, true>, sm)) != cudaSuccess) return e;
-      k_xfwd<T, SRC_RESID, true, N, true><<<grid, 256, sm, st>>>(g, in, sc, slot, fdf, pdf, spec, rp, tw, lpb);
-    } else if (!g.top_open) {
-      if ((e = allow_smem(k_xfwd<T, SRC_RESID, false, 0>, sm)) != cudaSuccess) return e;
-      k_xfwd<T, SRC_RESID, false, 0><<<grid, 256, sm, st>>>(g, in, sc, slot, fdf, pdf, spec, rp, tw, lpb);
+      if (g.spec_planes) return cudaErrorInvalidValue;
+      if (src == SRC_F) return go(k_xfwd_rg<SRC_F, N, false>);
+      if (src == SRC_FDF) return go(k_xfwd_rg<SRC_FDF, N, false>);
+      if (!g.top_open) return go(k_xfwd_rg<SRC_RESID, N, false>);
+      return go(k_xfwd_rg<SRC_RESID, N, true>);
     } else {
-      if ((e = allow_smem(k_xfwd<T, SRC_RESID, false, 0, true>, sm)) != cudaSuccess) return e;
-      k_xfwd<T, SRC_RESID, false, 0, true><<<grid, 256, sm, st>>>(g, in, sc, slot, fdf, pdf, spec, rp, tw, lpb);
+      if (g.spec_planes) return cudaErrorInvalidValue;
+      if (src == SRC_F) return go_sm(k_xfwd<T, SRC_F, true, N>);
+      if (src == SRC_FDF) return go_sm(k_xfwd<T, SRC_FDF, true, N>);
+      if (do_fft && !g.top_open) return go_sm(k_xfwd<T, SRC_RESID, true, N>);
+      if (do_fft) return go_sm(k_xfwd<T, SRC_RESID, true, N, true>);
+      if (!g.top_open) return go_sm(k_xfwd<T, SRC_RESID, false, 0>);
+      return go_sm(k_xfwd<T, SRC_RESID, false, 0, true>);
     }
-    return cudaGetLastError();
   });
 }
 
@@ -1320,32 +1320,31 @@ template <typename T>
 cudaError_t launch_zfft(bool inverse, const GridDev& g, cpx<T>* spec, const RadixPlan& rp, const cpx<T>* tw,
                         int tkx, const DevScalars* sc, DevScalars* fin, cudaStream_t st) {
   const int nxh = g.nx / 2 + 1;
-  const int grid = g.ny * ((nxh + tkx - 1) / tkx);
-  const size_t sm = zfft_smem<T>(g.nz, tkx);
   return with_len<T>(g.nz, [&](auto NC) -> cudaError_t {
     constexpr int N = decltype(NC)::value;
-    cudaError_t e;
-    if constexpr (has_ct_lengths<T>::value && rgfft::is_rg<N>::value) {
-      const int L = rg_lines<N>(tkx);
+    if constexpr (has_ct_lengths<T>::value && (sizeof(T) == 4 ? has_rg<N>::value : rgfft::is_rg<N>::value)) {
+      using RP = z_plan<T, N>;
+      const int L = rg_lines<RP>(tkx);
       const int gr = g.ny * ((nxh + L - 1) / L);
       const size_t smr = rg_smem<T>(N, L);
-      if (inverse) {
-        if ((e = allow_smem(k_zfft_rg<T, true, N>, smr)) != cudaSuccess) return e;
-        launch_pdl(k_zfft_rg<T, true, N>, gr, L * (N / 16), smr, st, g, spec, tw, L, sc, fin);
-      } else {
-        if ((e = allow_smem(k_zfft_rg<T, false, N>, smr)) != cudaSuccess) return e;
-        launch_pdl(k_zfft_rg<T, false, N>, gr, L * (N / 16), smr, st, g, spec, tw, L, sc, fin);
-      }
-      return cudaGetLastError();
-    }
-    if (inverse) {
-      if ((e = allow_smem(k_zfft<T, true, N>, sm)) != cudaSuccess) return e;
-      k_zfft<T, true, N><<<grid, 256, sm, st>>>(g, spec, rp, tw, tkx, sc, fin);
+      auto go = [&](auto kernel) -> cudaError_t {
+        cudaError_t e = allow_smem(kernel, smr);
+        if (e != cudaSuccess) return e;
+        launch_pdl(kernel, gr, L * RP::T, smr, st, g, spec, tw, L, sc, fin);
+        return cudaGetLastError();
+      };
+      return inverse ? go(k_zfft_rg<T, true, N>) : go(k_zfft_rg<T, false, N>);
     } else {
-      if ((e = allow_smem(k_zfft<T, false, N>, sm)) != cudaSuccess) return e;
-      k_zfft<T, false, N><<<grid, 256, sm, st>>>(g, spec, rp, tw, tkx, sc, fin);
+      const int grid = g.ny * ((nxh + tkx - 1) / tkx);
+      const size_t sm = zfft_smem<T>(g.nz, tkx);
+      auto go = [&](auto kernel) -> cudaError_t {
+        cudaError_t e = allow_smem(kernel, sm);
+        if (e != cudaSuccess) return e;
+        launch_pdl(kernel, grid, 256, sm, st, g, spec, rp, tw, tkx, sc, fin);
+        return cudaGetLastError();
+      };
+      return inverse ? go(k_zfft<T, true, N>) : go(k_zfft<T, false, N>);
     }
-    return cudaGetLastError();
   });
 }
 
@@ -1354,7 +1353,7 @@ cudaError_t launch_ythomas(const GridDev& g, cpx<T>* spec, const T* tab, const i
                            const DevScalars* sc, cudaStream_t st) {
   const int nxh = g.nx / 2 + 1;
   const dim3 grid((nxh + 127) / 128, g.nz);
-  k_ythomas<T><<<grid, 128, 0, st>>>(g, spec, tab, off, len, a, sc);
+  launch_pdl(k_ythomas<T>, grid, 128, 0, st, g, spec, tab, off, len, a, sc);
   return cudaGetLastError();
 }
 
@@ -1363,33 +1362,31 @@ cudaError_t launch_ydct(const GridDev& g, cpx<T>* spec, const RadixPlan& rp, con
                         const T* lam_x, const T* lam_y, const T* lam_z, int tky, const DevScalars* zsc,
                         cudaStream_t st) {
   const int nxh = g.nx / 2 + 1;
-  const int grid = g.nz * ((nxh + tky - 1) / tky);
-  const size_t sm = zfft_smem<T>(g.ny, tky);
   return with_len<T>(g.ny, [&](auto NC) -> cudaError_t {
     constexpr int N = decltype(NC)::value;
     // (FP32 only: the register-staged y pass in pairs needs ~190 registers, one
     // CTA per SM, and ran 1.6x slower than the shared-memory form at 256^3)
-    if constexpr (sizeof(T) == 4 && rgfft::is_rg<N>::value) {
-      const int L = rg_lines<N>(tky);
+    if constexpr (sizeof(T) == 4 && has_rg<N>::value) {
+      using RP = rgfft::plan_for<N>;
+      const int L = rg_lines<RP>(tky);
       const int gr = g.nz * ((nxh + L - 1) / L);
       const size_t smr = rg_smem<T>(N, L);
-      if constexpr (N == 256 && sizeof(T) == 4) {
-        cudaError_t e = allow_smem(k_ydct256, smr);
+      auto go = [&](auto kernel) -> cudaError_t {
+        cudaError_t e = allow_smem(kernel, smr);
         if (e != cudaSuccess) return e;
-        launch_pdl(k_ydct256, gr, L * (N / 16), smr, st, g, (cpx<float>*)spec, (const cpx<float>*)tw,
-                                                 (const cpx<float>*)wq, (const float*)lam_x, (const float*)lam_y,
-                                                 (const float*)lam_z, L, zsc);
+        launch_pdl(kernel, gr, L * RP::T, smr, st, g, spec, tw, wq, lam_x, lam_y, lam_z, L, zsc);
         return cudaGetLastError();
-      }
-      cudaError_t e = allow_smem(k_ydct_rg<T, N>, smr);
+      };
+      if constexpr (N == 256) return go(k_ydct256);
+      else return go(k_ydct_rg<T, N>);
+    } else {
+      const int grid = g.nz * ((nxh + tky - 1) / tky);
+      const size_t sm = zfft_smem<T>(g.ny, tky);
+      cudaError_t e = allow_smem(k_ydct<T, N>, sm);
       if (e != cudaSuccess) return e;
-      launch_pdl(k_ydct_rg<T, N>, gr, L * (N / 16), smr, st, g, spec, tw, wq, lam_x, lam_y, lam_z, L, zsc);
+      launch_pdl(k_ydct<T, N>, grid, 256, sm, st, g, spec, rp, tw, wq, lam_x, lam_y, lam_z, tky, zsc);
       return cudaGetLastError();
     }
-    cudaError_t e = allow_smem(k_ydct<T, N>, sm);
-    if (e != cudaSuccess) return e;
-    k_ydct<T, N><<<grid, 256, sm, st>>>(g, spec, rp, tw, wq, lam_x, lam_y, lam_z, tky, zsc);
-    return cudaGetLastError();
   });
 }
 
@@ -1400,49 +1397,50 @@ cudaError_t launch_xinv(int mode, const GridDev& g, const cpx<T>* spec, double* 
   const int nlines = g.ny * g.nz;
   const int grid = (nlines + lpb - 1) / lpb;
   const size_t sm = xinv_smem<T>(g.nx, lpb);
+  auto go_sm = [&](auto kernel) -> cudaError_t {  // the shared-memory form
+    cudaError_t e = allow_smem(kernel, sm);
+    if (e != cudaSuccess) return e;
+    launch_pdl(kernel, grid, 256, sm, st, g, spec, p, pdf, scale, rp, tw, lpb, sc, psc);
+    return cudaGetLastError();
+  };
   return with_len<T>(g.nx / 2, [&](auto NC) -> cudaError_t {
     constexpr int N = decltype(NC)::value;
-    cudaError_t e;
-    // (the register-staged form writes an FP64 p with 16-byte stores)
-    if constexpr (sizeof(T) == 4 && rgfft::is_rg<N>::value) {
-      if (mode != XI_F64 || ((uintptr_t)p & 15u) == 0 || g.spec_planes) {
+    if constexpr (sizeof(T) == 4 && has_rg<N>::value) {
+      // (the register-staged form writes an FP64 p with 16-byte stores; a solve
+      // of this type leaves p in pairs, so no caller's p gets here)
       if (mode == XI_F64 && ((uintptr_t)p & 15u) != 0) return cudaErrorMisalignedAddress;
-      const int L = rg_xlines<N>(lpb);
+      using RP = rgfft::plan_for<N>;
+      const int L = rg_lines<RP>(lpb);
       const int gr = (nlines + L - 1) / L;
       const size_t smr = xrg_smem(g.nx, L, g.spec_planes != 0);
       auto go = [&](auto kernel) -> cudaError_t {
         cudaError_t e2 = allow_smem(kernel, smr);
         if (e2 != cudaSuccess) return e2;
-        launch_pdl(kernel, gr, L * (N / 16), smr, st, g, (const cpx<float>*)spec, p, pdf, scale, (const cpx<float>*)tw, L,
-                                               sc, psc, p32);
+        launch_pdl(kernel, gr, L * RP::T, smr, st, g, (const cpx<float>*)spec, p, pdf, scale, (const cpx<float>*)tw, L,
+                   sc, psc, p32);
         return cudaGetLastError();
       };
-      if (mode == XI_F32 && !(p32 && is_pow2_scale(g))) return cudaErrorInvalidValue;
-      if (g.spec_planes) {
-        if (mode == XI_F64) return go(k_xinv_rg<XI_F64, N, true>);
-        if (mode == XI_DF) return go(k_xinv_rg<XI_DF, N, true>);
-        if (mode == XI_F32) return go(k_xinv_rg<XI_F32, N, true>);
-        return go(k_xinv_rg<XI_DF_ACC, N, true>);
+      if constexpr (rgfft::is_rg<N>::value) {  // (the plane layout and the FP32 p: powers of two)
+        if (mode == XI_F32 && !(p32 && is_pow2_scale(g))) return cudaErrorInvalidValue;
+        if (g.spec_planes) {
+          if (mode == XI_F64) return go(k_xinv_rg<XI_F64, N, true>);
+          if (mode == XI_DF) return go(k_xinv_rg<XI_DF, N, true>);
+          if (mode == XI_F32) return go(k_xinv_rg<XI_F32, N, true>);
+          return go(k_xinv_rg<XI_DF_ACC, N, true>);
+        }
+        if (mode == XI_F32) return go(k_xinv_rg<XI_F32, N>);
       }
+      if (g.spec_planes || mode == XI_F32) return cudaErrorInvalidValue;
       if (mode == XI_F64) return go(k_xinv_rg<XI_F64, N>);
       if (mode == XI_DF) return go(k_xinv_rg<XI_DF, N>);
-      if (mode == XI_F32) return go(k_xinv_rg<XI_F32, N>);
       return go(k_xinv_rg<XI_DF_ACC, N>);
-      }
-    }
-    if (mode == XI_F32 || p32) return cudaErrorInvalidValue;  // FP32 p: the register-staged passes only
-    if (g.spec_planes) return cudaErrorInvalidValue;  // plane layout: power-of-two nx/2 only
-    if (mode == XI_F64) {
-      if ((e = allow_smem(k_xinv<T, XI_F64, N>, sm)) != cudaSuccess) return e;
-      k_xinv<T, XI_F64, N><<<grid, 256, sm, st>>>(g, spec, p, pdf, scale, rp, tw, lpb, sc, psc);
-    } else if (mode == XI_DF) {
-      if ((e = allow_smem(k_xinv<T, XI_DF, N>, sm)) != cudaSuccess) return e;
-      k_xinv<T, XI_DF, N><<<grid, 256, sm, st>>>(g, spec, p, pdf, scale, rp, tw, lpb, sc, psc);
     } else {
-      if ((e = allow_smem(k_xinv<T, XI_DF_ACC, N>, sm)) != cudaSuccess) return e;
-      k_xinv<T, XI_DF_ACC, N><<<grid, 256, sm, st>>>(g, spec, p, pdf, scale, rp, tw, lpb, sc, psc);
+      if (mode == XI_F32 || p32) return cudaErrorInvalidValue;  // FP32 p: the register-staged passes only
+      if (g.spec_planes) return cudaErrorInvalidValue;          // plane layout: power-of-two nx/2 only
+      if (mode == XI_F64) return go_sm(k_xinv<T, XI_F64, N>);
+      if (mode == XI_DF) return go_sm(k_xinv<T, XI_DF, N>);
+      return go_sm(k_xinv<T, XI_DF_ACC, N>);
     }
-    return cudaGetLastError();
   });
 }
 
