@@ -346,7 +346,7 @@ size_t rhs_smem(int nx, int ny, int lines) {
 // Planes per CTA of the column-stack form at S = 2.  A CTA marches kc planes
 // after a prologue worth about one and a half; with N CTAs on `slots` resident
 // places the march takes (N / slots + 1/2) (kc + 3/2) steps, and where one wave
-// holds them all, kc + 3/2 steps that are the shorter the emptier the SMs
+// holds them all, kc + 3/2 longer steps, the shorter the emptier the SMs
 // (measured over kc = 1 .. 32 at 32^3 .. 384 x 256 x 384: within 4 % of the best
 // of each, except 12 % on 48 x 192 x 32; the fixed kc = 8 before cost 32^3 24
 // instead of 10 us, 64^3 24 instead of 14).
@@ -360,7 +360,7 @@ int rhs_planes(int nx, int ny, int nz) {
   double least = 0.0;
   for (int kc = 1; kc <= 12 && kc <= nz; ++kc) {
     const double w = ntile * ((nz + kc - 1) / kc) / slots;
-    const double t = (w <= 1.0 ? 0.45 + 0.55 * w : w + 0.5) * (kc + 1.5);
+    const double t = (w <= 1.0 ? 0.75 + 0.7 * w : w + 0.5) * (kc + 1.5);
     if (kc == 1 || t < least) {
       least = t;
       best = kc;
@@ -428,7 +428,12 @@ cudaError_t launch_rhs(const GridDev& g, const StencilIn& in, DevScalars* sc, do
   if (g.nx <= kRhsStackNx) {
     // column-stack form: tj is the stack height S
     const int threads = stack_threads(g.nx, launch_stacks(g.nx, g.ny, tj));
-    auto go = [&](auto kernel) { launch_pdl(kernel, grid, threads, sm, st, g, in, sc, o, kc); };
+    cudaError_t e = cudaSuccess;
+    auto go = [&](auto kernel) {
+      // (instances near 48 KB and beyond opt in where they are launched: a plan has one)
+      if (sm > kSmemOptIn) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+      if (e == cudaSuccess) e = launch_pdl(kernel, grid, threads, sm, st, g, in, sc, o, kc);
+    };
     switch (tj) {
       case 1: stack_kernel<1>(g.nx, threads, in.face_rule, proj, go); break;
       case 2: stack_kernel<2>(g.nx, threads, in.face_rule, proj, go); break;
@@ -436,10 +441,14 @@ cudaError_t launch_rhs(const GridDev& g, const StencilIn& in, DevScalars* sc, do
       case 8: stack_kernel<8>(g.nx, threads, in.face_rule, proj, go); break;
       default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
   }
   const int cpt = tj * g.nx <= 4 * kRhsThreads ? 4 : 8;
-  auto go = [&](auto kernel) { launch_pdl(kernel, grid, kRhsThreads, sm, st, g, in, sc, o, tj, kc); };
+  cudaError_t e = cudaSuccess;
+  auto go = [&](auto kernel) {
+    if (sm > kSmemOptIn) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e == cudaSuccess) e = launch_pdl(kernel, grid, kRhsThreads, sm, st, g, in, sc, o, tj, kc);
+  };
   // instance table: [cpt][rule][proj]
 #define PPE_RHS_CASE(C)                                                        \
   if (cpt == C) {                                                              \
@@ -452,72 +461,21 @@ cudaError_t launch_rhs(const GridDev& g, const StencilIn& in, DevScalars* sc, do
   PPE_RHS_CASE(4)
   PPE_RHS_CASE(8)
 #undef PPE_RHS_CASE
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
-
-namespace {
-// Opt-in dynamic shared memory of one instance: the per-CTA maximum minus the
-// instance's static shared memory (the reduction scratch).
-template <typename K>
-cudaError_t raise_smem(K kernel, size_t* dyn_max) {
-  cudaFuncAttributes a;
-  cudaError_t e = cudaFuncGetAttributes(&a, kernel);
-  if (e != cudaSuccess) return e;
-  const size_t cap = kSmemPerCta - a.sharedSizeBytes;
-  if (dyn_max && cap < *dyn_max) *dyn_max = cap;
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap);
-}
-}  // namespace
 
 cudaError_t launch_finish_sums(const GridDev& g, DevScalars* sc, cudaStream_t st) {
   launch_pdl(k_finish_sums, 1, 256, 0, st, g, sc);
   return cudaGetLastError();
 }
 
-namespace {
-template <int C>
-cudaError_t raise_march(size_t* cap) {
-  cudaError_t e = raise_smem(k_rhs_march<C, 0, true>, cap);
-  if (e == cudaSuccess) e = raise_smem(k_rhs_march<C, 0, false>, cap);
-  if (e == cudaSuccess) e = raise_smem(k_rhs_march<C, 1, true>, cap);
-  if (e == cudaSuccess) e = raise_smem(k_rhs_march<C, 1, false>, cap);
-  return e;
-}
-template <int S>
-cudaError_t raise_stack(size_t* cap) {
-  cudaError_t e = cudaSuccess;
-  auto up = [&](auto kernel) {
-    if (e == cudaSuccess) e = raise_smem(kernel, cap);
-  };
-  // every width with an instance of its own, and one thread count per block bound
-  for (int rule = 0; rule < 2; ++rule) {
-    for (int nx : {32, 64, 96, 128, 192, 256, 384}) stack_kernel<S>(nx, 256, rule, true, up);
-    for (int threads : {256, 384, 512}) {
-      stack_kernel<S>(8, threads, rule, true, up);
-      stack_kernel<S>(8, threads, rule, false, up);
-    }
-  }
-  return e;
-}
-cudaError_t raise_all(size_t* cap) {
-  cudaError_t e = raise_march<4>(cap);
-  if (e == cudaSuccess) e = raise_march<8>(cap);
-  if (e == cudaSuccess) e = raise_stack<1>(cap);
-  if (e == cudaSuccess) e = raise_stack<2>(cap);
-  if (e == cudaSuccess) e = raise_stack<4>(cap);
-  if (e == cudaSuccess) e = raise_stack<8>(cap);
-  return e;
-}
-}  // namespace
-
-cudaError_t set_rhs_smem_limit() {
-  size_t cap = kSmemPerCta;
-  return raise_all(&cap);
-}
-
-size_t rhs_smem_limit() {
-  size_t cap = kSmemPerCta;
-  return raise_all(&cap) == cudaSuccess ? cap : 0;
+// The per-CTA maximum minus an instance's static shared memory (the reduction
+// scratch, the same in every instance of a form).
+size_t rhs_smem_limit(int nx) {
+  cudaFuncAttributes a;
+  const cudaError_t e = nx <= kRhsStackNx ? cudaFuncGetAttributes(&a, k_rhs_stack<1, 0, false, 256, 0>)
+                                          : cudaFuncGetAttributes(&a, k_rhs_march<4, 0, false>);
+  return e == cudaSuccess ? kSmemPerCta - a.sharedSizeBytes : 0;
 }
 
 }  // namespace ppe

@@ -1,24 +1,18 @@
 // Programmatic dependent launch of the projection's kernel chain.
 //
-// Each kernel of the step is launched with programmatic stream serialisation:
-// it may be scheduled while the kernel before it on the stream is still
-// running (its CTAs take the SM slots that the earlier kernel's last wave
-// leaves free, and its launch latency overlaps that kernel's tail).  Every such
-// kernel begins with pdl_enter(): griddepcontrol.wait blocks until the
-// preceding kernel has completed and its memory operations are visible (so no
-// global data is read before it), then griddepcontrol.launch_dependents lets
-// the next kernel be scheduled in turn.  Because the trigger follows the wait,
-// at most one kernel ahead of the running one is ever resident and waiting,
-// and a kernel sees everything every earlier kernel wrote (each completed
-// after the wait of its successor's predecessor returned).  Launched without
-// the attribute, both instructions have no effect.
-//
-// Launches into a stream that is being captured into a graph take no
-// attribute: in the batched graph (independent per-plan branches running side
-// by side) the waiting CTAs held slots the other branches could use (64 grids:
-// 4.74 -> 4.94 ms per batch with the attribute), and within one plan's
-// refinement graph it changed nothing measurable.  On direct launches it saves
-// about 1 us per kernel boundary (256^3 step: 1.121 -> 1.105 ms).
+// Each kernel of the step is launched with programmatic stream serialisation
+// and begins with pdl_enter(): griddepcontrol.wait blocks until the preceding
+// kernel has completed and its memory operations are visible, so no global
+// data is read before it.  No kernel signals its dependents early: the implicit
+// trigger when its CTAs exit lets the next kernel's launch overlap the end of
+// this one and its memory flush, which is most of a launch's cost (chain of
+// small kernels: 1.4 against 4.1 us each).  An explicit trigger at the start
+// (griddepcontrol.launch_dependents) packed the next kernel's CTAs into the few
+// SM slots free at that moment, under the running kernel's shared-memory
+// carve-out: few CTAs ended up several to an SM, and passes with many loads in
+// flight kept a small L1 (128^3: 222 -> 205 us without it, 64^3 FP64 81 -> 65,
+// 96^3 153 -> 144, 256^3 FP64 1238 -> 1206).  Captured launches take the same
+// attribute (64-grid batch 3960 -> 3930 us, 32^3's refinement graph 74 -> 72).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -28,17 +22,13 @@ namespace ppe {
 
 __device__ __forceinline__ void pdl_enter() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // kernel<<<grid, block, smem, st>>>(args...), with programmatic stream
-// serialisation unless st is capturing (see above); returns the launch's error.
+// serialisation (in a capture: a programmatic edge); returns the launch's error.
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                        Args&&... args) {
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  const cudaError_t ce = cudaStreamIsCapturing(st, &cs);
-  if (ce != cudaSuccess) return ce;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
@@ -48,7 +38,7 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cfg.attrs = at;
-  cfg.numAttrs = cs == cudaStreamCaptureStatusNone ? 1 : 0;
+  cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 

@@ -906,17 +906,14 @@ ppe_status ppe_plan(ppe_plan_t* out, const ppe_grid* g, const ppe_options* opt, 
         s = make_thomas<float>(P);
         P->yscan_ok = s == PPE_OK;
       }
-      if (s == PPE_OK) s = cuda_status(set_smem_limits<float>());
     } else if (P->pairs) {
       s = make_twiddles<dd>(&P->tw_x, g->nx);
       if (s == PPE_OK) s = make_twiddles<dd>(&P->tw_z, g->nz);
       if (s == PPE_OK) s = make_dct_tables<dd>(P);
-      if (s == PPE_OK) s = cuda_status(set_smem_limits<dd>());
     } else {
       s = make_twiddles<double>(&P->tw_x, g->nx);
       if (s == PPE_OK) s = make_twiddles<double>(&P->tw_z, g->nz);
       if (s == PPE_OK) s = make_thomas<double>(P);
-      if (s == PPE_OK) s = cuda_status(set_smem_limits<double>());
     }
   }
   // the plane-layout schedules where their kernels exist (and, for the fused
@@ -1024,7 +1021,7 @@ ppe_status ppe_set_tuning(ppe_plan_t P, const ppe_tuning* t) {
   auto pow2 = [](int v, int lo, int hi) { return v >= lo && v <= hi && (v & (v - 1)) == 0; };
   const size_t lim = 227 * 1024;
   const int nx = P->g.nx, ny = P->g.ny, nz = P->g.nz;
-  if (!pow2(t->rhs_lines, 1, 8) || rhs_smem(nx, ny, t->rhs_lines) > rhs_smem_limit() ||
+  if (!pow2(t->rhs_lines, 1, 8) || rhs_smem(nx, ny, t->rhs_lines) > rhs_smem_limit(nx) ||
       t->rhs_lines > rhs_max_lines(nx))
     return PPE_ERR_INVALID_ARG;
   if (t->rhs_planes < 1 || t->rhs_planes > nz) return PPE_ERR_INVALID_ARG;

@@ -120,9 +120,10 @@ size_t rhs_smem(int nx, int ny, int lines);  // dynamic shared memory of the RHS
 int rhs_tile_lines(int nx, int ny, int lines);  // lines per CTA
 int rhs_planes(int nx, int ny, int nz);         // z planes per CTA, chosen for the grid
 int rhs_max_lines(int nx);  // largest rhs_lines value (lines per thread stack, or per tile when nx > 512)
-cudaError_t set_rhs_smem_limit();
-size_t rhs_smem_limit();  // largest dynamic shared memory every k_rhs_march instance accepts
+size_t rhs_smem_limit(int nx);  // largest dynamic shared memory an instance of this nx accepts
 constexpr size_t kSmemPerCta = 227 * 1024;  // opt-in shared memory per CTA (static + dynamic)
+// dynamic shared memory above which a kernel opts in (48 KB less the static scratch of a kernel)
+constexpr size_t kSmemOptIn = 44 * 1024;
 
 // ---- unsplit projection (k_pcg.cu) ----
 // Constants of the variable-coefficient operator as pairs: 1/h^2, 1/h, 1/dt, dt h.
@@ -186,8 +187,6 @@ template <typename T>
 size_t zfft_smem(int nz, int tkx);
 template <typename T>
 size_t xinv_smem(int nx, int lpb);
-template <typename T>
-cudaError_t set_smem_limits();
 template <typename T>
 size_t xpass_smem_limit();  // largest dynamic shared memory of the x passes (static scratch excluded)
 template <typename T>

@@ -91,10 +91,10 @@ cudaError_t with_len(int n, F&& f) {
   return f(std::integral_constant<int, 0>{});
 }
 
-// Kernels needing more than the default 48 KB of dynamic shared memory opt in.
+// Kernels needing more than the default 48 KB of shared memory opt in.
 template <typename K>
 cudaError_t allow_smem(K kernel, size_t bytes) {
-  if (bytes <= 48 * 1024) return cudaSuccess;
+  if (bytes <= kSmemOptIn) return cudaSuccess;
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
@@ -504,11 +504,22 @@ __device__ __forceinline__ void zfft_body(GridDev g, cpx<T>* spec, RadixPlan rp,
     if (kx0 + c < nxh) spec[base + k * rowstride + c] = r[idx];
   }
 }
+// With fin the grid has one CTA more, the first, which only totals the partial
+// sums (finish_sums) beside the others: done by the CTA of the first tile, the
+// sums' latency (loads, trees, two FP64 divisions) preceded its transform and
+// the z pass of a small grid waited for it (32^3: 10 -> 4 us, 96^3: 10 -> 4).
+__device__ __forceinline__ bool finish_cta(DevScalars* fin, const GridDev& g) {
+  if (!fin || blockIdx.x != 0) return false;
+  finish_sums(fin, g);
+  return true;
+}
 template <typename T, bool INV, int N>
 __global__ void __launch_bounds__(256) k_zfft(GridDev g, cpx<T>* spec, RadixPlan rp, const cpx<T>* __restrict__ tw,
                                               int tkx, const DevScalars* sc, DevScalars* fin) {
   pdl_enter();
-  zfft_body<T, INV, N>(g, spec, rp, tw, tkx, sc, fin, blockIdx.x, gridDim.x);
+  if (finish_cta(fin, g)) return;
+  const uint32_t extra = fin ? 1u : 0u;
+  zfft_body<T, INV, N>(g, spec, rp, tw, tkx, sc, nullptr, blockIdx.x - extra, gridDim.x - extra);
 }
 
 // Register-staged z pass (FP32, nz a length with a plan, and pairs, nz a power
@@ -547,7 +558,9 @@ template <typename T, bool INV, int N>
 __global__ void __launch_bounds__(rgfft::max_threads<z_plan<T, N>>()) k_zfft_rg(GridDev g, cpx<T>* spec, const cpx<T>* __restrict__ tw, int L,
                                                  const DevScalars* sc, DevScalars* fin) {
   pdl_enter();
-  zfft_rg_body<T, INV, N, z_plan<T, N>>(g, spec, tw, L, sc, fin, blockIdx.x, gridDim.x);
+  if (finish_cta(fin, g)) return;
+  const uint32_t extra = fin ? 1u : 0u;
+  zfft_rg_body<T, INV, N, z_plan<T, N>>(g, spec, tw, L, sc, nullptr, blockIdx.x - extra, gridDim.x - extra);
 }
 
 // ---------------------------------------------------------------------------
@@ -1259,11 +1272,6 @@ size_t zpass_smem_limit() {
 }
 
 template <typename T>
-cudaError_t set_smem_limits() {
-  return set_rhs_smem_limit();
-}
-
-template <typename T>
 cudaError_t launch_xfwd(int src, bool do_fft, const GridDev& g, const StencilIn& in, DevScalars* sc, int slot,
                         df* fdf, const df* pdf, cpx<T>* spec, const RadixPlan& rp, const cpx<T>* tw, int lpb,
                         cudaStream_t st) {
@@ -1325,7 +1333,7 @@ cudaError_t launch_zfft(bool inverse, const GridDev& g, cpx<T>* spec, const Radi
     if constexpr (has_ct_lengths<T>::value && (sizeof(T) == 4 ? has_rg<N>::value : rgfft::is_rg<N>::value)) {
       using RP = z_plan<T, N>;
       const int L = rg_lines<RP>(tkx);
-      const int gr = g.ny * ((nxh + L - 1) / L);
+      const int gr = g.ny * ((nxh + L - 1) / L) + (fin ? 1 : 0);
       const size_t smr = rg_smem<T>(N, L);
       auto go = [&](auto kernel) -> cudaError_t {
         cudaError_t e = allow_smem(kernel, smr);
@@ -1335,7 +1343,7 @@ cudaError_t launch_zfft(bool inverse, const GridDev& g, cpx<T>* spec, const Radi
       };
       return inverse ? go(k_zfft_rg<T, true, N>) : go(k_zfft_rg<T, false, N>);
     } else {
-      const int grid = g.ny * ((nxh + tkx - 1) / tkx);
+      const int grid = g.ny * ((nxh + tkx - 1) / tkx) + (fin ? 1 : 0);
       const size_t sm = zfft_smem<T>(g.nz, tkx);
       auto go = [&](auto kernel) -> cudaError_t {
         cudaError_t e = allow_smem(kernel, sm);
@@ -1448,7 +1456,6 @@ cudaError_t launch_xinv(int mode, const GridDev& g, const cpx<T>* spec, double* 
   template size_t xfwd_smem<T>(int, int);                                                                        \
   template size_t zfft_smem<T>(int, int);                                                                        \
   template size_t xinv_smem<T>(int, int);                                                                        \
-  template cudaError_t set_smem_limits<T>();                                                                     \
   template size_t xpass_smem_limit<T>();                                                                         \
   template cudaError_t launch_xfwd<T>(int, bool, const GridDev&, const StencilIn&, DevScalars*, int, df*,       \
                                       const df*, cpx<T>*, const RadixPlan&, const cpx<T>*, int, cudaStream_t);  \

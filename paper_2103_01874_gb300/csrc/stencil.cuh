@@ -212,33 +212,67 @@ __device__ __forceinline__ void sum_parts_fixed(const double2* part, int n, doub
 
 // Totals of the per-CTA partial sums of the current call, formed by one CTA
 // (all threads) in a kernel that runs after their producers (the kernel
-// boundary orders the accesses): the sum of f from the forward x transform
-// (sum_parts_fixed over its CTAs) and the wall flux from the wall tiles of
-// k_rhs_march (chunk by chunk, lower wall then upper wall).
+// boundary orders the accesses): the sum of f from the forward x transform,
+// the sum of p from the inverse one and the wall flux from the wall tiles of
+// the right-hand side (lower and upper wall of each chunk of planes).  The
+// three totals share one pass of loads and one tree, in an order that depends
+// only on their counts and blockDim.x (thread t takes t, t + blockDim.x, ... in
+// turn): a dependent loop over the chunks and two trees one after the other
+// held the z pass of a small grid back (32^3: 10 us of it).
 __device__ __forceinline__ void finish_sums(DevScalars* sc, const GridDev& g) {
+  __shared__ double red_f[3][32];
   const size_t nynz = (size_t)g.ny * g.nz;
-  const int xp = sc->x_parts;
-  const int pp = sc->p_parts;
-  double fs = 0.0, ps = 0.0, unused;
-  if (xp > 0) sum_parts_fixed(sc->part + nynz, xp, &fs, &unused);
-  __syncthreads();  // thread 0 has read the first reduction's shared scratch
+  const double2* const part = sc->part;
+  const int xp = sc->x_parts, pp = sc->p_parts, nt = sc->rhs_tiles, nc = sc->rhs_chunks;
+  const int wp = nt > 0 ? (nt > 1 ? 2 * nc : nc) : 0;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  auto walls = [&](int i) -> const double2* {  // chunk by chunk, lower then upper wall
+    return nt > 1 ? part + (size_t)(i >> 1) * nt + (i & 1) * (nt - 1) : part + i;
+  };
+  double v[3] = {0.0, 0.0, 0.0};
+  const int most = max(xp, max(pp, wp));
+  constexpr int U = 2;  // loads issued before their additions (the order is unchanged; more cost the z pass registers)
+  for (int i0 = threadIdx.x; i0 < most; i0 += U * blockDim.x) {
+    double a[U][3];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int i = i0 + u * blockDim.x;
+      a[u][0] = i < xp ? __ldcg(&part[nynz + i].x) : 0.0;
+      a[u][1] = i < pp ? __ldcg(&part[2 * nynz + i].x) : 0.0;
+      a[u][2] = i < wp ? __ldcg(&walls(i)->x) : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int i = i0 + u * blockDim.x;
+      if (i < xp) v[0] += a[u][0];
+      if (i < pp) v[1] += a[u][1];
+      if (i < wp) v[2] += a[u][2];
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+    for (int q = 0; q < 3; ++q) v[q] += __shfl_down_sync(0xffffffffu, v[q], o);
+  }
+  if (lane == 0) {
+#pragma unroll
+    for (int q = 0; q < 3; ++q) red_f[q][wid] = v[q];
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  for (int w = 1; w < nw; ++w) {
+#pragma unroll
+    for (int q = 0; q < 3; ++q) v[q] += red_f[q][w];
+  }
+  const double fs = v[0], ps = v[1];
   // the sum of the p the last inverse x transform formed: the next correction's
   // zero mode is -sum(p)/ny, which adds -mean(p) to p after the inverse transforms
   // (DCT-III unscaled in its zero mode, z and x inverses scaled by 1/(nx nz))
-  if (pp > 0) sum_parts_fixed(sc->part + 2 * nynz, pp, &ps, &unused);
-  if (threadIdx.x != 0) return;
   if (pp > 0) {
     sc->zmode = -ps / (double)g.ny;
     sc->p_parts = 0;
   }
-  const int nt = sc->rhs_tiles, nc = sc->rhs_chunks;
   if (nt > 0) {
-    double ws = 0.0;
-    for (int c = 0; c < nc; ++c) {
-      ws += sc->part[(size_t)c * nt].x;
-      if (nt > 1) ws += sc->part[(size_t)c * nt + nt - 1].x;
-    }
-    sc->wall_flux = ws;
+    sc->wall_flux = v[2];
     sc->rhs_ran = 1;
   }
   if (xp > 0) {
