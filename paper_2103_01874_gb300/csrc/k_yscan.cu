@@ -1,4 +1,5 @@
-// y pass of the FP32 solve with walls as a tridiagonal solve in scan form.
+// y pass of the FP32 solve as a tridiagonal solve in scan form (a choice with
+// walls; the form of an open top).
 #include "pdl.cuh"
 #include "ppe_internal.h"
 
@@ -6,8 +7,7 @@ namespace ppe {
 
 namespace {
 
-// y pass of the FP32 solve with walls as the tridiagonal (Thomas) solve of
-// k_ythomas, written as two affine scans so that a line is shared by 16
+// y pass of the FP32 solve as the tridiagonal (Thomas) solve of k_ythomas, written as two affine scans so that a line is shared by 16
 // threads.  Per (kx, kz) line the forward elimination is the recurrence
 // xt_j = (d_j - a xt_{j-1}) m_j = alpha_j xt_{j-1} + beta_j (alpha_j = -a m_j,
 // beta_j = d_j m_j) and the back substitution x_j = xt_j - a m_j x_{j+1}; both
@@ -119,8 +119,8 @@ __global__ void __launch_bounds__(256, (S <= 4 ? 4 : (S == 8 ? 3 : (S == 16 ? 2 
   const bool valid = kx < nxh;
   const int j0 = t * S;
   cpx<float>* col = spec + (size_t)kz * ny * nxh + kx;
-  const bool singular = kz == 0 && kx == 0;  // (column 0 of the CTA kz = 0, kx0 = 0)
-  const bool sing_cta = kz == 0 && kx0 == 0;  // uniform over the CTA
+  const bool singular = !g.top_open && kz == 0 && kx == 0;  // (column 0 of the CTA kz = 0, kx0 = 0)
+  const bool sing_cta = !g.top_open && kz == 0 && kx0 == 0;  // uniform over the CTA
   if (sing_cta) singular_line(spec, ny, nxh, (double)a, zsc ? zsc->zmode : 0.0, sline, sx, sy);  // (kz = kx = 0)
   int off = 0, J = 0;
   float m_inf = 0.0f, m_last = 0.0f;

@@ -61,6 +61,9 @@ struct ppe_plan_s {
   // y step of the LEGACY schedule (ppe_tuning.y_solve): PPE_Y_TRIDIAGONAL where
   // yscan_ok (FP32_REFINE, walls, ny <= 512: Thomas tables built)
   bool yscan_ok;
+  // an open top in FP32, ny <= 512: the scan form (128 x 192 x 128: 65 -> 29 us per y
+  // pass against one thread per line, whose serial chains fill no SM)
+  bool yscan_open;
   int y_solve;
   alignas(64) CUtensorMap tmap;
   alignas(64) CUtensorMap tmap_z;
@@ -447,7 +450,7 @@ ppe_status solve_tail(ppe_plan_t P, int mode, double* p64, df* pdf, bool guarded
   }
   PPE_LAUNCH(P, K_ZFFT_FWD,
              launch_zfft<T>(false, P->gd, spec, P->rp_z, (const cpx<T>*)P->tw_z, P->tkx, sc, fin, P->stream));
-  if (P->y_solve == PPE_Y_TRIDIAGONAL) {  // (FP32, walls) the Thomas elimination in scan form
+  if (P->y_solve == PPE_Y_TRIDIAGONAL || P->yscan_open) {  // (FP32) the Thomas elimination in scan form
     PPE_LAUNCH(P, K_YTHOMAS, launch_ythomas_scan(P->gd, (cpx<float>*)spec, (const float*)P->tab, P->line_off,
                                                  P->line_len, (float)P->a_y, P->sc, P->stream));
   } else if ((P->fp32 || P->pairs) && !P->gd.top_open) {  // DCT-II/III for walls; the open top: tridiagonal solve
@@ -902,6 +905,7 @@ ppe_status ppe_plan(ppe_plan_t* out, const ppe_grid* g, const ppe_options* opt, 
       if (s == PPE_OK) s = make_twiddles<float>(&P->tw_z, g->nz);
       if (s == PPE_OK) s = P->gd.top_open ? make_thomas<float>(P) : make_dct_tables<float>(P);
       // walls: the multipliers of the tridiagonal y method too (PPE_Y_TRIDIAGONAL)
+      P->yscan_open = P->gd.top_open && yscan_elems(g->ny) > 0;
       if (s == PPE_OK && !P->gd.top_open && yscan_elems(g->ny) > 0) {
         s = make_thomas<float>(P);
         P->yscan_ok = s == PPE_OK;
