@@ -16,7 +16,10 @@
 // Vectors are float pairs (dfloat.cuh); K uses per-face coefficients
 // a_f = 1 / (rho_f h^2) formed once per call.  Dot products are reduced per
 // CTA in pairs and totalled in a fixed order by one-CTA scalar kernels.
+#include <algorithm>
+
 #include "dfloat.cuh"
+#include "pdl.cuh"
 #include "ppe_internal.h"
 #include "stencil.cuh"
 
@@ -33,6 +36,10 @@ __device__ __forceinline__ CellIdx cell_of(const GridDev& g, uint32_t c) {
   const uint32_t k = fdiv(r, g.fd_ny);
   return {c, c - r * (uint32_t)g.nx, r - k * (uint32_t)g.ny, k};
 }
+
+// CTAs of a vector kernel per SM (64 registers a thread), and so the partial
+// sums that the scalar kernels total
+constexpr int kVcCtas = 4;
 
 // 1 / (rho_f h^2) of the face between cells of densities a, b
 template <int RULE>
@@ -51,6 +58,7 @@ __global__ void __launch_bounds__(256) k_vc_setup(GridDev g, const double* __res
                                                   const double* __restrict__ S, const double* __restrict__ rho,
                                                   VcConst C, df* ax, df* ay, df* az, df* r, DevScalars* sc,
                                                   double2* part) {
+  pdl_enter();
   const uint32_t nx = g.nx, ny = g.ny, nz = g.nz, plane = nx * ny, n = plane * nz;
   df gsum = {0.0f, 0.0f};
   float gmax = 0.0f;
@@ -78,6 +86,7 @@ __global__ void __launch_bounds__(256) k_vc_setup(GridDev g, const double* __res
 
 // One CTA: mean of g, and the iteration state.
 __global__ void k_vc_start(GridDev g, DevScalars* sc, const double2* part, int nparts, double tol, int max_iter) {
+  pdl_enter();
   double gs, unused;
   sum_parts_fixed(part, nparts, &gs, &unused);
   if (threadIdx.x != 0) return;
@@ -95,34 +104,51 @@ __global__ void k_vc_start(GridDev g, DevScalars* sc, const double2* part, int n
   sc->pcg_cont = 1;
 }
 
-// Kp = K p and the CTA's part of p . Kp
-__global__ void __launch_bounds__(256) k_vc_apply(GridDev g, const df* __restrict__ p, const df* __restrict__ ax,
-                                                  const df* __restrict__ ay, const df* __restrict__ az, df* Kp,
-                                                  double2* part) {
-  const uint32_t nx = g.nx, ny = g.ny, nz = g.nz, plane = nx * ny, n = plane * nz;
+// Kp = K p and the CTA's part of p . Kp.  Like the other vector kernels of an
+// iteration it takes two cells of a line per thread (nx is even) with 16-byte
+// accesses, on one resident wave of CTAs: bound by load latency, one cell per
+// thread in 1.6 waves took 21 us at 128^3 where the 84 MB lie in L2.
+__global__ void __launch_bounds__(256, kVcCtas) k_vc_apply(GridDev g, const df* __restrict__ p,
+                                                           const df* __restrict__ ax, const df* __restrict__ ay,
+                                                           const df* __restrict__ az, df* Kp, double2* part) {
+  pdl_enter();
+  const uint32_t nx = g.nx, ny = g.ny, nz = g.nz, m = nx / 2, plane = nx * ny, n2 = m * ny * nz;
   df dot = {0.0f, 0.0f};
-  for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x) {
-    const CellIdx q = cell_of(g, c);
-    const uint32_t xm = (q.i == 0) ? c + nx - 1 : c - 1, xp = (q.i + 1 == nx) ? c + 1 - nx : c + 1;
-    const uint32_t zm = (q.k == 0) ? c + (nz - 1) * plane : c - plane;
-    const uint32_t zp = (q.k + 1 == nz) ? c - (nz - 1) * plane : c + plane;
-    const df pc = p[c];
+  for (uint32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < n2; q += gridDim.x * blockDim.x) {
+    const uint32_t line = fdiv(q, g.fd_m), e = q - line * m;
+    const uint32_t k = fdiv(line, g.fd_ny), j = line - k * ny;
+    const uint32_t c = 2 * q;
+    const uint32_t zm = (k == 0) ? c + (nz - 1) * plane : c - plane;
+    const uint32_t zp = (k + 1 == nz) ? c - (nz - 1) * plane : c + plane;
+    const uint32_t xp = (e + 1 == m) ? c + 2 - nx : c + 2;
+    auto two = [](const df* a, uint32_t o) { return *reinterpret_cast<const float4*>(a + o); };
+    const float4 P = two(p, c), Zm = two(p, zm), Zp = two(p, zp);
+    const float4 Ym = j > 0 ? two(p, c - nx) : P, Yp = j + 1 < ny ? two(p, c + nx) : P;  // (no difference: no flux)
+    const df pm = p[(e == 0) ? c + nx - 1 : c - 1], pp = p[xp], axp = ax[xp];
+    const float4 AX = two(ax, c), AY = two(ay, c), AYp = two(ay, j + 1 < ny ? c + nx : c), AZ = two(az, c),
+                 AZp = two(az, zp);
+    const df p0 = {P.x, P.y}, p1 = {P.z, P.w};
     // sum over the faces of a_f (p_c - p_nbr); the wall faces carry no flux
-    df acc = df_mulz(ax[c], df_subz(pc, p[xm]));
-    acc = df_addz(acc, df_mulz(ax[xp], df_subz(pc, p[xp])));
-    acc = df_addz(acc, df_mulz(az[c], df_subz(pc, p[zm])));
-    acc = df_addz(acc, df_mulz(az[zp], df_subz(pc, p[zp])));
-    if (q.j > 0) acc = df_addz(acc, df_mulz(ay[c], df_subz(pc, p[c - nx])));
-    if (q.j + 1 < ny) acc = df_addz(acc, df_mulz(ay[c + nx], df_subz(pc, p[c + nx])));
-    const df kp = df_norm(acc);
-    Kp[c] = kp;
-    dot = df_addz(dot, df_mulz(pc, kp));
+    const df mid = df_mulz(df{AX.z, AX.w}, df_subz(p0, p1));
+    df a0 = df_addz(df_mulz(df{AX.x, AX.y}, df_subz(p0, pm)), mid);
+    df a1 = df_subz(df_mulz(axp, df_subz(p1, pp)), mid);
+    a0 = df_addz(a0, df_mulz(df{AZ.x, AZ.y}, df_subz(p0, df{Zm.x, Zm.y})));
+    a1 = df_addz(a1, df_mulz(df{AZ.z, AZ.w}, df_subz(p1, df{Zm.z, Zm.w})));
+    a0 = df_addz(a0, df_mulz(df{AZp.x, AZp.y}, df_subz(p0, df{Zp.x, Zp.y})));
+    a1 = df_addz(a1, df_mulz(df{AZp.z, AZp.w}, df_subz(p1, df{Zp.z, Zp.w})));
+    a0 = df_addz(a0, df_mulz(df{AY.x, AY.y}, df_subz(p0, df{Ym.x, Ym.y})));
+    a1 = df_addz(a1, df_mulz(df{AY.z, AY.w}, df_subz(p1, df{Ym.z, Ym.w})));
+    a0 = df_norm(df_addz(a0, df_mulz(df{AYp.x, AYp.y}, df_subz(p0, df{Yp.x, Yp.y}))));
+    a1 = df_norm(df_addz(a1, df_mulz(df{AYp.z, AYp.w}, df_subz(p1, df{Yp.z, Yp.w}))));
+    *reinterpret_cast<float4*>(Kp + c) = make_float4(a0.hi, a0.lo, a1.hi, a1.lo);
+    dot = df_addz(df_addz(dot, df_mulz(p0, a0)), df_mulz(p1, a1));
   }
   block_pair_sums(dot, df{0.0f, 0.0f}, part + blockIdx.x);
 }
 
 // One CTA: alpha = rz / (p . K p)
 __global__ void k_vc_alpha(DevScalars* sc, const double2* part, int nparts) {
+  pdl_enter();
   double pkp, unused;
   sum_parts_fixed(part, nparts, &pkp, &unused);
   if (threadIdx.x != 0) return;
@@ -130,30 +156,42 @@ __global__ void k_vc_alpha(DevScalars* sc, const double2* part, int nparts) {
 }
 
 // x += alpha p, r -= alpha Kp; max |r - mean(g)| (r keeps the mean of g, which
-// K p and the solve do not change)
-__global__ void __launch_bounds__(256) k_vc_update(uint32_t n, df* x, df* r, const df* __restrict__ p,
-                                                   const df* __restrict__ Kp, DevScalars* sc) {
+// K p and the solve do not change).  n2 pairs of cells.
+__global__ void __launch_bounds__(256, kVcCtas) k_vc_update(uint32_t n2, float4* x, float4* r,
+                                                            const float4* __restrict__ p,
+                                                            const float4* __restrict__ Kp, DevScalars* sc) {
+  pdl_enter();
   const df a = d2df(sc->pcg_alpha);
   const df gm = sc->pcg_gmean_df;
   float rmax = 0.0f;
-  for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x) {
-    x[c] = df_norm(df_addz(x[c], df_mulz(a, p[c])));
-    const df rn = df_norm(df_subz(r[c], df_mulz(a, Kp[c])));
-    r[c] = rn;
-    rmax = fmaxf(rmax, fabsf(df_to_f(df_subz(rn, gm))));
+  auto axpy = [&](df v, df w) { return df_norm(df_addz(v, df_mulz(a, w))); };
+  auto less = [&](df v, df w) {
+    const df o = df_norm(df_subz(v, df_mulz(a, w)));
+    rmax = fmaxf(rmax, fabsf(df_to_f(df_subz(o, gm))));
+    return o;
+  };
+  for (uint32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < n2; q += gridDim.x * blockDim.x) {
+    const float4 X = x[q], R = r[q], P = p[q], K = Kp[q];
+    const df x0 = axpy(df{X.x, X.y}, df{P.x, P.y}), x1 = axpy(df{X.z, X.w}, df{P.z, P.w});
+    const df r0 = less(df{R.x, R.y}, df{K.x, K.y}), r1 = less(df{R.z, R.w}, df{K.z, K.w});
+    x[q] = make_float4(x0.hi, x0.lo, x1.hi, x1.lo);
+    r[q] = make_float4(r0.hi, r0.lo, r1.hi, r1.lo);
   }
   block_max_to(&sc->pcg_rmax_bits, rmax);
 }
 
 // The CTA's parts of r . z and z . K p, with z = -zs (zs = L^{-1} r from the
 // FFT solve)
-__global__ void __launch_bounds__(256) k_vc_dots(uint32_t n, const df* __restrict__ r, const df* __restrict__ zs,
-                                                 const df* __restrict__ Kp, double2* part) {
+__global__ void __launch_bounds__(256, kVcCtas) k_vc_dots(uint32_t n2, const float4* __restrict__ r,
+                                                          const float4* __restrict__ zs,
+                                                          const float4* __restrict__ Kp, double2* part) {
+  pdl_enter();
   df d1 = {0.0f, 0.0f}, d2 = {0.0f, 0.0f};
-  for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x) {
-    const df z = zs[c];
-    d1 = df_addz(d1, df_mulz(r[c], z));
-    d2 = df_addz(d2, df_mulz(z, Kp[c]));
+  for (uint32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < n2; q += gridDim.x * blockDim.x) {
+    const float4 R = r[q], Z = zs[q], K = Kp[q];
+    const df z0 = {Z.x, Z.y}, z1 = {Z.z, Z.w};
+    d1 = df_addz(df_addz(d1, df_mulz(df{R.x, R.y}, z0)), df_mulz(df{R.z, R.w}, z1));
+    d2 = df_addz(df_addz(d2, df_mulz(z0, df{K.x, K.y})), df_mulz(z1, df{K.z, K.w}));
   }
   block_pair_sums(df_neg(d1), df_neg(d2), part + blockIdx.x);
 }
@@ -162,6 +200,7 @@ __global__ void __launch_bounds__(256) k_vc_dots(uint32_t n, const df* __restric
 // condition of the iteration graph when use_handle.
 __global__ void k_vc_beta(DevScalars* sc, const double2* part, int nparts, int first,
                           cudaGraphConditionalHandle handle, int use_handle) {
+  pdl_enter();
   double rz, zkp;
   sum_parts_fixed(part, nparts, &rz, &zkp);
   if (threadIdx.x != 0) return;
@@ -182,11 +221,16 @@ __global__ void k_vc_beta(DevScalars* sc, const double2* part, int nparts, int f
 }
 
 // p = z + beta p = beta p - zs
-__global__ void __launch_bounds__(256) k_vc_pupdate(uint32_t n, df* p, const df* __restrict__ zs,
-                                                    const DevScalars* sc) {
+__global__ void __launch_bounds__(256, kVcCtas) k_vc_pupdate(uint32_t n2, float4* p, const float4* __restrict__ zs,
+                                                             const DevScalars* sc) {
+  pdl_enter();
   const df b = d2df(sc->pcg_beta);
-  for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x)
-    p[c] = df_norm(df_subz(df_mulz(b, p[c]), zs[c]));
+  for (uint32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < n2; q += gridDim.x * blockDim.x) {
+    const float4 P = p[q], Z = zs[q];
+    const df p0 = df_norm(df_subz(df_mulz(b, df{P.x, P.y}), df{Z.x, Z.y}));
+    const df p1 = df_norm(df_subz(df_mulz(b, df{P.z, P.w}), df{Z.z, Z.w}));
+    p[q] = make_float4(p0.hi, p0.lo, p1.hi, p1.lo);
+  }
 }
 
 // The CTA's part of sum x; then one CTA forms the mean.  The FFT preconditioner
@@ -194,12 +238,14 @@ __global__ void __launch_bounds__(256) k_vc_pupdate(uint32_t n, df* p, const df*
 // (FP32: ~1e-8 of max |x|); p is returned with zero mean, as Eq. (30) fixes
 // p only up to a constant.
 __global__ void __launch_bounds__(256) k_vc_sum(uint32_t n, const df* __restrict__ x, double2* part) {
+  pdl_enter();
   df s = {0.0f, 0.0f};
   for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x) s = df_addz(s, x[c]);
   block_pair_sums(s, df{0.0f, 0.0f}, part + blockIdx.x);
 }
 
 __global__ void k_vc_xmean(DevScalars* sc, const double2* part, int nparts, double n) {
+  pdl_enter();
   double xs, unused;
   sum_parts_fixed(part, nparts, &xs, &unused);
   if (threadIdx.x == 0) sc->pcg_xmean_df = d2df(xs / n);
@@ -213,6 +259,7 @@ __global__ void __launch_bounds__(256) k_vc_correct(GridDev g, const double* __r
                                                     const df* __restrict__ ay, const df* __restrict__ az, VcConst C,
                                                     const DevScalars* sc, double* p_out, double* u_out,
                                                     double* v_out, double* w_out) {
+  pdl_enter();
   const uint32_t nx = g.nx, ny = g.ny, nz = g.nz, plane = nx * ny;
   const df xm0 = sc->pcg_xmean_df;
   const uint32_t total = nz * (ny + 1) * nx;
@@ -241,12 +288,15 @@ __global__ void __launch_bounds__(256) k_vc_correct(GridDev g, const double* __r
 // launchers
 // ---------------------------------------------------------------------------
 namespace {
+// one resident wave (less where the cells do not fill it)
 unsigned flat_grid(size_t n) {
-  size_t b = (n + 255) / 256;
-  const size_t cap = (size_t)152 * 8;
+  size_t b = (n / 2 + 255) / 256;
+  const size_t cap = (size_t)152 * kVcCtas;
   if (b > cap) b = cap;
   return (unsigned)(b ? b : 1);
 }
+const float4* f4(const df* p) { return reinterpret_cast<const float4*>(p); }
+float4* f4(df* p) { return reinterpret_cast<float4*>(p); }
 }  // namespace
 
 unsigned vc_grid(size_t n) { return flat_grid(n); }
@@ -256,53 +306,53 @@ cudaError_t launch_vc_setup(const GridDev& g, int rule, const double* u, const d
                             DevScalars* sc, double2* part, cudaStream_t st) {
   const unsigned grid = flat_grid((size_t)g.nx * g.ny * g.nz);
   if (rule == 0)
-    k_vc_setup<0><<<grid, 256, 0, st>>>(g, u, v, w, S, rho, C, ax, ay, az, r, sc, part);
+    launch_pdl(k_vc_setup<0>, grid, 256, 0, st, g, u, v, w, S, rho, C, ax, ay, az, r, sc, part);
   else
-    k_vc_setup<1><<<grid, 256, 0, st>>>(g, u, v, w, S, rho, C, ax, ay, az, r, sc, part);
+    launch_pdl(k_vc_setup<1>, grid, 256, 0, st, g, u, v, w, S, rho, C, ax, ay, az, r, sc, part);
   return cudaGetLastError();
 }
 
 cudaError_t launch_vc_start(const GridDev& g, DevScalars* sc, const double2* part, double tol, int max_iter,
                             cudaStream_t st) {
   const int nparts = (int)flat_grid((size_t)g.nx * g.ny * g.nz);
-  k_vc_start<<<1, 256, 0, st>>>(g, sc, part, nparts, tol, max_iter);
+  launch_pdl(k_vc_start, 1, 256, 0, st, g, sc, part, nparts, tol, max_iter);
   return cudaGetLastError();
 }
 
 cudaError_t launch_vc_apply(const GridDev& g, const df* p, const df* ax, const df* ay, const df* az, df* Kp,
                             double2* part, cudaStream_t st) {
-  k_vc_apply<<<flat_grid((size_t)g.nx * g.ny * g.nz), 256, 0, st>>>(g, p, ax, ay, az, Kp, part);
+  launch_pdl(k_vc_apply, flat_grid((size_t)g.nx * g.ny * g.nz), 256, 0, st, g, p, ax, ay, az, Kp, part);
   return cudaGetLastError();
 }
 
 cudaError_t launch_vc_alpha(const GridDev& g, DevScalars* sc, const double2* part, cudaStream_t st) {
-  k_vc_alpha<<<1, 256, 0, st>>>(sc, part, (int)flat_grid((size_t)g.nx * g.ny * g.nz));
+  launch_pdl(k_vc_alpha, 1, 256, 0, st, sc, part, (int)flat_grid((size_t)g.nx * g.ny * g.nz));
   return cudaGetLastError();
 }
 
 cudaError_t launch_vc_update(const GridDev& g, df* x, df* r, const df* p, const df* Kp, DevScalars* sc,
                              cudaStream_t st) {
   const size_t n = (size_t)g.nx * g.ny * g.nz;
-  k_vc_update<<<flat_grid(n), 256, 0, st>>>((uint32_t)n, x, r, p, Kp, sc);
+  launch_pdl(k_vc_update, flat_grid(n), 256, 0, st, (uint32_t)(n / 2), f4(x), f4(r), f4(p), f4(Kp), sc);
   return cudaGetLastError();
 }
 
 cudaError_t launch_vc_dots(const GridDev& g, const df* r, const df* zs, const df* Kp, double2* part,
                            cudaStream_t st) {
   const size_t n = (size_t)g.nx * g.ny * g.nz;
-  k_vc_dots<<<flat_grid(n), 256, 0, st>>>((uint32_t)n, r, zs, Kp, part);
+  launch_pdl(k_vc_dots, flat_grid(n), 256, 0, st, (uint32_t)(n / 2), f4(r), f4(zs), f4(Kp), part);
   return cudaGetLastError();
 }
 
 cudaError_t launch_vc_beta(const GridDev& g, DevScalars* sc, const double2* part, int first,
                            cudaGraphConditionalHandle handle, int use_handle, cudaStream_t st) {
-  k_vc_beta<<<1, 256, 0, st>>>(sc, part, (int)flat_grid((size_t)g.nx * g.ny * g.nz), first, handle, use_handle);
+  launch_pdl(k_vc_beta, 1, 256, 0, st, sc, part, (int)flat_grid((size_t)g.nx * g.ny * g.nz), first, handle, use_handle);
   return cudaGetLastError();
 }
 
 cudaError_t launch_vc_pupdate(const GridDev& g, df* p, const df* zs, const DevScalars* sc, cudaStream_t st) {
   const size_t n = (size_t)g.nx * g.ny * g.nz;
-  k_vc_pupdate<<<flat_grid(n), 256, 0, st>>>((uint32_t)n, p, zs, sc);
+  launch_pdl(k_vc_pupdate, flat_grid(n), 256, 0, st, (uint32_t)(n / 2), f4(p), f4(zs), sc);
   return cudaGetLastError();
 }
 
@@ -312,10 +362,10 @@ cudaError_t launch_vc_correct(const GridDev& g, const double* u, const double* v
                               cudaStream_t st) {
   const size_t n = (size_t)g.nx * g.ny * g.nz;
   const unsigned gs = flat_grid(n);
-  k_vc_sum<<<gs, 256, 0, st>>>((uint32_t)n, x, part);
-  k_vc_xmean<<<1, 256, 0, st>>>(sc, part, (int)gs, (double)n);
+  launch_pdl(k_vc_sum, gs, 256, 0, st, (uint32_t)n, x, part);
+  launch_pdl(k_vc_xmean, 1, 256, 0, st, sc, part, (int)gs, (double)n);
   const size_t total = (size_t)g.nx * (g.ny + 1) * g.nz;
-  k_vc_correct<<<flat_grid(total), 256, 0, st>>>(g, u, v, w, x, ax, ay, az, C, sc, p_out, u_out, v_out, w_out);
+  launch_pdl(k_vc_correct, (unsigned)std::min<size_t>((total + 255) / 256, (size_t)152 * 8), 256, 0, st, g, u, v, w, x, ax, ay, az, C, sc, p_out, u_out, v_out, w_out);
   return cudaGetLastError();
 }
 
