@@ -497,6 +497,29 @@ using plan_for = typename std::conditional<has_split<N>::value, SplitPlan<N>, Re
 template <class RP>
 constexpr int max_threads() { return RP::T > 32 ? 512 : 256; }
 
+// the thread's asynchronous copies to shared memory (async.cuh)
+__device__ __forceinline__ void copies_landed() {
+#ifdef __CUDA_ARCH__
+  asm volatile("cp.async.wait_all;\n" ::: "memory");
+#endif
+}
+
+// A loader in two phases: fetch(e) issues the loads of element e and make(raw,
+// e) forms its value.  The first pass fetches up to eight elements before it
+// makes the first: with the arithmetic of a value between its loads and the
+// next element's, the compiler left few loads in flight and the x passes
+// waited for one after the other (long scoreboard 8.6 of 19 cycles per
+// instruction).
+template <class F, class M>
+struct TwoPhase {
+  F fetch;
+  M make;
+};
+template <class F, class M>
+__device__ __forceinline__ TwoPhase<F, M> two_phase(F f, M m) { return {f, m}; }
+template <class L> struct is_two_phase : std::false_type {};
+template <class F, class M> struct is_two_phase<TwoPhase<F, M>> : std::true_type {};
+
 // LD_SHARED: ld reads the shared buffer (the first pass then waits for all
 // reads before writing); later passes always read all before their stores.
 template <typename T, bool INV, class RP, int S, int TWS, bool LD_SHARED, int PAD, class Ld, class St>
@@ -509,11 +532,23 @@ __device__ __forceinline__ void pass(Ld& ld, St& st, cpx<T>* ln, int es, int t0,
   for (int it = 0; it < IT; ++it) {
     const int t = t0 + it * TPL;
     if (NB % TPL != 0 && t >= NB) continue;
+    if constexpr (S == 0 && is_two_phase<Ld>::value) {
+      constexpr int B = R < 8 ? R : 8;
+      decltype(ld.fetch(0)) raw[B];
 #pragma unroll
-    for (int q = 0; q < R; ++q) {
-      const int e = t + q * NB;
-      if (S == 0) v[it][q] = ld(e);
-      else v[it][q] = ln[rowp<PAD>(e) * es];
+      for (int q0 = 0; q0 < R; q0 += B) {
+#pragma unroll
+        for (int q = q0; q < q0 + B && q < R; ++q) raw[q - q0] = ld.fetch(t + q * NB);
+#pragma unroll
+        for (int q = q0; q < q0 + B && q < R; ++q) v[it][q] = ld.make(raw[q - q0], t + q * NB);
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < R; ++q) {
+        const int e = t + q * NB;
+        if constexpr (S == 0) v[it][q] = ld(e);
+        else v[it][q] = ln[rowp<PAD>(e) * es];
+      }
     }
   }
   if (S > 0 || LD_SHARED) __syncthreads();  // in place: every read of the pass before any write
@@ -539,6 +574,7 @@ __device__ __forceinline__ void pass(Ld& ld, St& st, cpx<T>* ln, int es, int t0,
       else ln[rowp<PAD>(o + q * NS) * es] = v[it][q];
     }
   }
+  if (S == 0) copies_landed();  // (a twiddle table copied to shared memory behind the first pass's loads)
   if (S + 1 < NST) __syncthreads();
 }
 
@@ -554,7 +590,7 @@ __device__ __forceinline__ void run_from(Ld& ld, St& st, cpx<T>* ln, int es, int
 // thread of the CTA calls; t0 in [0, RP::T) is the thread's rank within its
 // line).  `tw` holds exp(-2 pi i t/(N*TWS)) and must be visible to all threads
 // before the second pass (the barrier after the first pass suffices when it is
-// written before the call).  The caller synchronises after the call before
+// written or its asynchronous copies are issued before the call).  The caller synchronises after the call before
 // reusing the buffer.
 template <typename T, bool INV, class RP, int TWS, bool LD_SHARED, int PAD = PAD_ROWS, class Ld, class St>
 __device__ __forceinline__ void run_plan(Ld&& ld, St&& st, cpx<T>* ln, int es, int t0, const cpx<T>* __restrict__ tw) {

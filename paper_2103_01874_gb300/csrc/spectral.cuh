@@ -303,7 +303,7 @@ __device__ __forceinline__ void xfwd_rg_body(GridDev g, StencilIn in, DevScalars
   const bool valid = line < nlines;
   cpx<T>* buf = reinterpret_cast<cpx<T>*>(smem_raw);  // L lines of LS
   cpx<T>* tws = buf + L * LS;                          // exp(-2 pi i t/nx), t < nx
-  for (int t = threadIdx.x; t < nx; t += blockDim.x) tws[t] = tw[t];
+  for (int t = threadIdx.x; t < nx; t += blockDim.x) cp_async<sizeof(cpx<T>)>(&tws[t], &tw[t]);
   const uint32_t c0 = line * (uint32_t)nx;  // 32-bit offsets (grids up to 1024^3)
   float vmax = 0.0f;
   df fsum = {0.0f, 0.0f};
@@ -328,13 +328,12 @@ __device__ __forceinline__ void xfwd_rg_body(GridDev g, StencilIn in, DevScalars
     // f as pairs, written by the right-hand-side kernel (which also took ||f||)
     const float4* fl = reinterpret_cast<const float4*>(fdf + c0);
     rgfft::run_plan<T, false, RP, 2, false>(
-        [&](int e) -> cpx<T> {
-          if (!valid) return {(T)0, (T)0};
-          const float4 q = fl[e];
-          const df v0 = {q.x, q.y}, v1 = {q.z, q.w};
-          fsum = df_addz(df_addz(fsum, v0), v1);
-          return {df_to_f(v0), df_to_f(v1)};
-        },
+        rgfft::two_phase([&](int e) { return valid ? fl[e] : make_float4(0.0f, 0.0f, 0.0f, 0.0f); },
+                         [&](float4 q, int) -> cpx<T> {
+                           const df v0 = {q.x, q.y}, v1 = {q.z, q.w};
+                           fsum = df_addz(df_addz(fsum, v0), v1);
+                           return {df_to_f(v0), df_to_f(v1)};
+                         }),
         put, buf + ll * LS, 1, t0, tws);
   } else {
     // residual r = f - L p in pairs, second differences as (p+ + p-) - 2 p
@@ -539,7 +538,7 @@ __device__ __forceinline__ void zfft_rg_body(GridDev g, cpx<T>* spec, const cpx<
   const uint32_t kx0 = (bid - j * ntile) * L;
   cpx<T>* buf = reinterpret_cast<cpx<T>*>(smem_raw);
   cpx<T>* tws = buf + rgfft::rows(N) * L;  // exp(-2 pi i t/nz)
-  for (int t = threadIdx.x; t < N; t += blockDim.x) tws[t] = tw[t];
+  for (int t = threadIdx.x; t < N; t += blockDim.x) cp_async<sizeof(cpx<T>)>(&tws[t], &tw[t]);
   const int line = threadIdx.x & (L - 1), t0 = threadIdx.x >> ilog2_dev(L);
   const bool valid = kx0 + line < nxh;
   const uint32_t rs = (uint32_t)g.ny * nxh;  // kz stride (32-bit offsets: spectra below 2^32 elements)
@@ -787,7 +786,7 @@ __device__ __forceinline__ void ydct_rg_body(GridDev g, cpx<T>* spec, const cpx<
   const uint32_t kz = bid / ntile, kx0 = (bid - kz * ntile) * L;
   cpx<T>* buf = reinterpret_cast<cpx<T>*>(smem_raw);
   cpx<T>* tws = buf + rgfft::rows(N) * L;  // exp(-2 pi i t/ny)
-  for (int t = threadIdx.x; t < N; t += blockDim.x) tws[t] = tw[t];
+  for (int t = threadIdx.x; t < N; t += blockDim.x) cp_async<sizeof(cpx<T>)>(&tws[t], &tw[t]);
   const int lg = ilog2_dev(L);
   const int line = threadIdx.x & (L - 1), t0 = threadIdx.x >> lg;
   const bool valid = kx0 + line < nxh;
@@ -876,7 +875,7 @@ __device__ __forceinline__ void ydct256_body(GridDev g, cpx<float>* spec, const 
   const uint32_t kz = bid / ntile, kx0 = (bid - kz * ntile) * L;
   cpx<T>* buf = reinterpret_cast<cpx<T>*>(smem_raw);
   cpx<T>* tws = buf + rgfft::rows(N) * L;  // exp(-2 pi i t/ny)
-  for (int t = threadIdx.x; t < N; t += blockDim.x) tws[t] = tw[t];
+  for (int t = threadIdx.x; t < N; t += blockDim.x) cp_async<sizeof(cpx<T>)>(&tws[t], &tw[t]);
   const int lg = ilog2_dev(L);
   const int line = threadIdx.x & (L - 1), t0 = threadIdx.x >> lg;  // t0 in [0, 16)
   const uint32_t kx = kx0 + line;
@@ -892,6 +891,7 @@ __device__ __forceinline__ void ydct256_body(GridDev g, cpx<float>* spec, const 
   SmallDft<T, false, 16>::run(v);
 #pragma unroll
   for (int q = 0; q < 16; ++q) ln[rgfft::row(16 * t0 + q) * L] = v[q];
+  cp_async_wait_all();
   __syncthreads();
   // forward pass 1: v[q] = X_{t0 + 16 q}
 #pragma unroll
@@ -1078,7 +1078,7 @@ __device__ __forceinline__ void xinv_rg_body(GridDev g, const cpx<float>* spec, 
   const bool valid = line < nlines;
   cpx<T>* buf = reinterpret_cast<cpx<T>*>(smem_raw);
   cpx<T>* tws = buf + L * LS;
-  for (int t = threadIdx.x; t < nx; t += blockDim.x) tws[t] = tw[t];
+  for (int t = threadIdx.x; t < nx; t += blockDim.x) cp_async<sizeof(cpx<T>)>(&tws[t], &tw[t]);
   if constexpr (PL) {
     const uint32_t l0 = bid * (uint32_t)L;
     const PlaneLanes pl = plane_lanes(L);
@@ -1113,17 +1113,21 @@ __device__ __forceinline__ void xinv_rg_body(GridDev g, const cpx<float>* spec, 
   const df sdf = d2df(scale);
   df psum = {0.0f, 0.0f};  // sum of the p written (pairs)
   // Z_k = E_k + i O_k, E = (X_k + conj X_{M-k})/2, O = (X_k - conj X_{M-k}) conj(W^k)/2
-  auto ld = [&](int k) -> cpx<T> {
-    if (!valid) return {(T)0, (T)0};
-    const cpx<T> xk = PL ? Xs[rgfft::row(k)] : X[k];
-    const cpx<T> xc = PL ? Xs[rgfft::row(M - k)] : X[M - k];
-    const cpx<T> e = {(T)0.5 * (xk.x + xc.x), (T)0.5 * (xk.y - xc.y)};
-    const cpx<T> dd = {(T)0.5 * (xk.x - xc.x), (T)0.5 * (xk.y + xc.y)};
-    cpx<T> w = tw[k];
-    w.y = -w.y;
-    const cpx<T> o = cmul(dd, w);
-    return {e.x - o.y, e.y + o.x};
+  struct Raw {
+    cpx<T> xk, xc, w;
   };
+  auto ld = rgfft::two_phase(
+      [&](int k) -> Raw {
+        if (PL) return {Xs[rgfft::row(k)], Xs[rgfft::row(M - k)], tw[k]};
+        if (!valid) return {{(T)0, (T)0}, {(T)0, (T)0}, tw[k]};
+        return {X[k], X[M - k], tw[k]};
+      },
+      [&](Raw r, int) -> cpx<T> {
+        const cpx<T> e = {(T)0.5 * (r.xk.x + r.xc.x), (T)0.5 * (r.xk.y - r.xc.y)};
+        const cpx<T> dd = {(T)0.5 * (r.xk.x - r.xc.x), (T)0.5 * (r.xk.y + r.xc.y)};
+        const cpx<T> o = cmul(dd, cpx<T>{r.w.x, -r.w.y});
+        return {e.x - o.y, e.y + o.x};
+      });
   auto st = [&](int n, cpx<T> v) {
     if (!valid) return;
     const uint32_t o = c0 + 2 * (uint32_t)n;
