@@ -88,44 +88,58 @@ __global__ void __launch_bounds__(256) k_correct_pre(GridDev g, double dt, const
 
 // Eq. (33) from the raw inputs:  u^{n+1} = u* - (dt/rho_0)(G p - beta_f G p_hat),
 // using 1/rho_f - 1/rho_0 = -beta_f/rho_0.  In-place (u_out == u) is allowed:
-// every thread reads u*, v*, w* only at the faces it writes.
+// every thread reads u*, v*, w* only at the faces it writes.  All of a thread's
+// inputs (the cell and its three lower neighbours, the three velocities) are
+// read before its first store: the outputs may alias the velocities, so loads
+// written after a store cannot move above it, and three rounds of latency per
+// cell were what the kernel waited for.
+template <int RULE>
 __global__ void __launch_bounds__(256) k_correct_full(GridDev g, StencilIn in, const DevScalars* sc, double* u_out,
                                                       double* v_out, double* w_out) {
   pdl_enter();
-  const size_t nx = (size_t)g.nx, ny = (size_t)g.ny;
-  const size_t total = (size_t)g.nz * (ny + 1) * nx;
+  const uint32_t nx = (uint32_t)g.nx, ny = (uint32_t)g.ny;
+  const uint32_t total = (uint32_t)g.nz * (ny + 1) * nx;
   const StencilConst K = sc->K;
-  const int rule = in.face_rule;
-  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total; t += (size_t)gridDim.x * blockDim.x) {
-    const uint32_t r = fdiv((uint32_t)t, g.fd_nx);
-    const int i = (int)((uint32_t)t - r * (uint32_t)nx);
+  for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
+    const uint32_t r = fdiv(t, g.fd_nx);
+    const int i = (int)(t - r * nx);
     const int k = (int)fdiv(r, g.fd_nyp1);
-    const int j = (int)(r - (uint32_t)k * (uint32_t)(ny + 1));
-    const size_t cv = t;
-    if (j == g.ny && g.top_open) {
+    const int j = (int)(r - (uint32_t)k * (ny + 1));
+    const double vs = in.v[t];
+    if (j == g.ny) {  // top face: a wall keeps v*
+      if (!g.top_open) {
+        v_out[t] = vs;
+        continue;
+      }
       // open top: the face between the top cell and its ghost (-p, -p_hat, same density)
-      const size_t ct = ((size_t)k * ny + (ny - 1)) * nx + i;
-      const df pt = d2df(in.p[ct]), ht = phat_df(in.pn, in.pnm1, ct), rt = d2df(__ldg(in.rho + ct));
-      const df b = beta_df(rt, rt, K, rule);
+      const uint32_t ct = ((uint32_t)k * ny + (ny - 1)) * nx + i;
+      const df pt = d2df(in.p[ct]), ht = phat_df(in.pn, in.pnm1, ct), rt = rho_cell<RULE>(d2df(__ldg(in.rho + ct)), K);
+      const df b = beta_cells<RULE, false>(rt, rt, K);
       const df gp = df_subz(df_neg(pt), pt), gh = df_subz(df_neg(ht), ht);
-      v_out[cv] = df2d(df_subz(d2df(in.v[cv]), df_mulz(K.gy, df_subz(gp, df_mulz(b, gh)))));
+      v_out[t] = df2d(df_subz(d2df(vs), df_mulz(K.gy, df_subz(gp, df_mulz(b, gh)))));
       continue;
     }
-    if (j == 0 || j == g.ny) {
-      v_out[cv] = in.v[cv];
-      if (j == g.ny) continue;
-    }
     const Nbr n = neighbours(g, i, j, k);
-    const df p0 = d2df(in.p[n.c]), h0 = phat_df(in.pn, in.pnm1, n.c), r0 = d2df(__ldg(in.rho + n.c));
-    auto face = [&](size_t cn, const df& gk) -> df {
-      const df b = beta_df(d2df(__ldg(in.rho + cn)), r0, K, rule);
-      const df gp = df_subz(p0, d2df(in.p[cn]));
-      const df gh = df_subz(h0, phat_df(in.pn, in.pnm1, cn));
-      return df_mulz(gk, df_subz(gp, df_mulz(b, gh)));
+    const size_t at[4] = {n.c, n.xm, j > 0 ? n.c - nx : n.c, n.zm};
+    double p[4], a[4], b[4], q[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      p[m] = in.p[at[m]];
+      a[m] = __ldg(in.pn + at[m]);
+      b[m] = __ldg(in.pnm1 + at[m]);
+      q[m] = __ldg(in.rho + at[m]);
+    }
+    const double us = in.u[n.c], ws = in.w[n.c];
+    const df p0 = d2df(p[0]), h0 = phat_of(a[0], b[0]), r0 = rho_cell<RULE>(d2df(q[0]), K);
+    auto corrected = [&](double v, int m, const df& gk) {
+      const df bf = beta_cells<RULE, false>(rho_cell<RULE>(d2df(q[m]), K), r0, K);
+      const df gp = df_subz(p0, d2df(p[m])), gh = df_subz(h0, phat_of(a[m], b[m]));
+      return df2d(df_subz(d2df(v), df_mulz(gk, df_subz(gp, df_mulz(bf, gh)))));
     };
-    if (j > 0) v_out[cv] = df2d(df_subz(d2df(in.v[cv]), face(n.c - nx, K.gy)));
-    u_out[n.c] = df2d(df_subz(d2df(in.u[n.c]), face(n.xm, K.gx)));
-    w_out[n.c] = df2d(df_subz(d2df(in.w[n.c]), face(n.zm, K.gz)));
+    const double un = corrected(us, 1, K.gx), vn = j > 0 ? corrected(vs, 2, K.gy) : vs, wn = corrected(ws, 3, K.gz);
+    u_out[n.c] = un;
+    v_out[t] = vn;
+    w_out[n.c] = wn;
   }
 }
 
@@ -258,7 +272,12 @@ cudaError_t launch_correct_pre(const GridDev& g, double dt, const df* upre, cons
 cudaError_t launch_correct_full(const GridDev& g, const StencilIn& in, const DevScalars* sc, double* u_out,
                                 double* v_out, double* w_out, cudaStream_t st) {
   const size_t total = (size_t)g.nz * (g.ny + 1) * g.nx;
-  launch_pdl(k_correct_full, grid_for(total, one_wave<k_correct_full>()), 256, 0, st, g, in, sc, u_out, v_out, w_out);
+  if (in.face_rule == 0)
+    launch_pdl(k_correct_full<0>, grid_for(total, one_wave<k_correct_full<0>>()), 256, 0, st, g, in, sc, u_out, v_out,
+               w_out);
+  else
+    launch_pdl(k_correct_full<1>, grid_for(total, one_wave<k_correct_full<1>>()), 256, 0, st, g, in, sc, u_out, v_out,
+               w_out);
   return cudaGetLastError();
 }
 

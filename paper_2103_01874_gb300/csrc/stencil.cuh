@@ -43,15 +43,7 @@ __device__ __forceinline__ StencilConst make_const(const GridDev& g, double rho0
   return K;
 }
 
-// beta_f = 1 - rho_0 / rho_f for the face between cells with densities a, b
-// (unnormalised pair; see the lazy operations in dfloat.cuh)
-__device__ __forceinline__ df beta_df(df a, df b, const StencilConst& K, int rule) {
-  const df one = {1.0f, 0.0f};
-  if (rule == 0) return df_subz(one, df_mulz(K.r02, df_recipz(df_addz(a, b))));   // 1 - 2 rho_0/(a+b)
-  return df_subz(one, df_mulz(K.r0h, df_addz(df_recipz(a), df_recipz(b))));        // 1 - (rho_0/2)(1/a+1/b)
-}
-
-// What the right-hand side keeps per cell for the face densities: rho itself
+// What a stencil keeps per cell for the face densities: rho itself
 // (arithmetic rule) or (rho_0/2)/rho (harmonic rule: beta_f is 1 minus the sum
 // of the two cells' values, so the reciprocal is taken once per cell instead
 // of at each of its six faces).
