@@ -302,8 +302,8 @@ __global__ void k_finish_sums(GridDev g, DevScalars* sc) {
 
 // Column-stack form of the march (rhs.cuh): one CTA of BT threads at most per
 // tile.  What bounds it: instruction issue and the latency of a step's loads
-// (493 warp instructions per 32 cells, 683 before; raw values prefetched into
-// shared memory, whole stacks per CTA).  256^3, projection outputs: 371 -> 305
+// (528 warp instructions per 32 cells, 683 before, at 71 % issue; raw values
+// prefetched into shared memory, whole stacks per CTA).  256^3, projection outputs: 371 -> 305
 // us (1.61 GB moved, 5.3 TB/s); 384 x 256 x 384 (the general march before):
 // 1248 -> 690; 192^3 (a quarter of the threads idle before): 201 -> 132; 128^3:
 // 66 -> 45.  The register budget (80 a thread for S <= 2: three CTAs of 256 threads
