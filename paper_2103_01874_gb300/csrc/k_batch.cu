@@ -481,7 +481,7 @@ __global__ void k_batch_cond(BatchCtl* ctl, cudaGraphConditionalHandle h) {
 }  // namespace
 
 cudaError_t batch_occupancy(size_t smem, int* ctas_per_sm) {
-  cudaError_t e = cudaFuncSetAttribute(k_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = allow_smem(k_batch, smem);
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, k_batch, kBatchThreads, smem);
 }

@@ -294,7 +294,7 @@ cudaError_t launch_zfft_tma(bool inverse, const GridDev& g, const CUtensorMap& t
     const int threads = jt * NZ / 16;  // 256 (fewer when ny < 4096 / nz)
     const size_t smem = 1024 + 2 * kPencilTile * sizeof(cpx<float>) + NZ * sizeof(cpx<float>) + 16;
     auto go = [&](auto kern) -> cudaError_t {
-      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      const cudaError_t e = allow_smem(kern, smem);
       if (e != cudaSuccess) return e;
       static int grid_cap = 0;  // resident CTAs of this instance (per process: one GPU model)
       if (!grid_cap) grid_cap = resident_ctas(kern, threads, smem);
@@ -315,7 +315,7 @@ cudaError_t launch_ydct_tma(const GridDev& g, cpx<float>* spec, const cpx<float>
     const size_t smem = 1024 + 2 * kPencilTile * sizeof(cpx<float>) + 2 * NY * sizeof(cpx<float>) +
                         NY * sizeof(float) + 16;
     auto kern = k_ydct_tma<NY>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(kern, smem);
     if (e != cudaSuccess) return e;
     static int grid_cap = 0;
     if (!grid_cap) grid_cap = resident_ctas(kern, threads, smem);

@@ -430,8 +430,7 @@ cudaError_t launch_rhs(const GridDev& g, const StencilIn& in, DevScalars* sc, do
     const int threads = stack_threads(g.nx, launch_stacks(g.nx, g.ny, tj));
     cudaError_t e = cudaSuccess;
     auto go = [&](auto kernel) {
-      // (instances near 48 KB and beyond opt in where they are launched: a plan has one)
-      if (sm > kSmemOptIn) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+      e = allow_smem(kernel, sm);
       if (e == cudaSuccess) e = launch_pdl(kernel, grid, threads, sm, st, g, in, sc, o, kc);
     };
     switch (tj) {
@@ -446,7 +445,7 @@ cudaError_t launch_rhs(const GridDev& g, const StencilIn& in, DevScalars* sc, do
   const int cpt = tj * g.nx <= 4 * kRhsThreads ? 4 : 8;
   cudaError_t e = cudaSuccess;
   auto go = [&](auto kernel) {
-    if (sm > kSmemOptIn) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    e = allow_smem(kernel, sm);
     if (e == cudaSuccess) e = launch_pdl(kernel, grid, kRhsThreads, sm, st, g, in, sc, o, tj, kc);
   };
   // instance table: [cpt][rule][proj]

@@ -201,7 +201,7 @@ cudaError_t go_zyz(const GridDev& g, const CUtensorMap& tmap, const cpx<float>* 
                    DevScalars* fin, cudaStream_t st, int* max_clusters) {
   using Cfg = ZyzCfg<NY, NZ>;
   auto kern = k_zyz<NY, NZ>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
+  cudaError_t e = allow_smem(kern, Cfg::SMEM);
   if (e != cudaSuccess) return e;
   const int nxh = g.nx / 2 + 1;
   cudaLaunchConfig_t cfg = {};

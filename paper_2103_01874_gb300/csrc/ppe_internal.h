@@ -124,6 +124,22 @@ size_t rhs_smem_limit(int nx);  // largest dynamic shared memory an instance of 
 constexpr size_t kSmemPerCta = 227 * 1024;  // opt-in shared memory per CTA (static + dynamic)
 // dynamic shared memory above which a kernel opts in (48 KB less the static scratch of a kernel)
 constexpr size_t kSmemOptIn = 44 * 1024;
+// Lets `kernel` be launched with `bytes` of dynamic shared memory.  The limit
+// belongs to the function in the whole process, so it only ever goes up, to all
+// that a CTA can have: one instance serves several sizes (the right-hand side's
+// nx = 128 takes 59,392 bytes at ny = 128 and 87,040 at ny = 96), and a limit set
+// to one launch's size would fail the launch of another host thread that had
+// set a larger one just before.
+template <typename K>
+cudaError_t allow_smem(K kernel, size_t bytes) {
+  if (bytes <= kSmemOptIn) return cudaSuccess;
+  cudaFuncAttributes a;
+  const cudaError_t e = cudaFuncGetAttributes(&a, kernel);
+  if (e != cudaSuccess) return e;
+  const int most = (int)(kSmemPerCta - a.sharedSizeBytes);
+  if (a.maxDynamicSharedSizeBytes >= most) return cudaSuccess;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
 
 // ---- unsplit projection (k_pcg.cu) ----
 // Constants of the variable-coefficient operator as pairs: 1/h^2, 1/h, 1/dt, dt h.

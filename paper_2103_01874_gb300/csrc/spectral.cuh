@@ -91,13 +91,6 @@ cudaError_t with_len(int n, F&& f) {
   return f(std::integral_constant<int, 0>{});
 }
 
-// Kernels needing more than the default 48 KB of shared memory opt in.
-template <typename K>
-cudaError_t allow_smem(K kernel, size_t bytes) {
-  if (bytes <= kSmemOptIn) return cudaSuccess;
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 // ---------------------------------------------------------------------------
 // forward x pass
 // ---------------------------------------------------------------------------
