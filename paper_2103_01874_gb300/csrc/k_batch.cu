@@ -55,7 +55,7 @@ bool len_ok(int n) {
     default: return false;
   }
 }
-bool pow2(int n) { return (n & (n - 1)) == 0; }
+constexpr bool pow2(int n) { return (n & (n - 1)) == 0; }
 unsigned cdiv(size_t a, size_t b) { return (unsigned)((a + b - 1) / b); }
 }  // namespace
 
@@ -79,10 +79,28 @@ namespace {
 // tiles of a transform pass along a length-n direction: 4096 / n lines for
 // power-of-two lengths, `cols` lines for radix-3 ones (256 threads share them:
 // BatchPlan)
-unsigned lines_per_tile(int n, int cols) { return pow2(n) ? 4096u / (unsigned)n : (unsigned)cols; }
+constexpr unsigned lines_per_tile(int n, int cols) { return pow2(n) ? 4096u / (unsigned)n : (unsigned)cols; }
+// Tiles of a radix-3 z or y pass that a CTA takes at once from an item's run:
+// as many as leave each line no fewer threads than its own kernel gives it.  A
+// tile alone has 16 threads a line in z and 32 in y for passes of 6 to 16
+// butterflies, and pays the call (the saved registers of the non-inlined pass are
+// more bytes than a 48-point tile): 16 grids of 128 x 48 x 128 take 1975 us one
+// tile at a time and 1616 so, 128 x 192 x 128 5662 and 5451; taking 96-point z
+// tiles two at a time, with 8 threads a line, is slower (3008 -> 3187).
+constexpr int tiles_at_once(int n, int cols) {
+  if (pow2(n)) return 1;
+  const int threads = n == 48 ? rgfft::plan_for<48>::T : n == 96 ? rgfft::plan_for<96>::T : rgfft::plan_for<192>::T;
+  int G = 1;
+  while (kBatchThreads / (2 * G * cols) >= threads) G *= 2;
+  return G;
+}
 constexpr size_t kRhoCellsPerTile = 65536;     // rho_0 reduction: 256 threads x 256 cells
 constexpr size_t kFacesPerThreadCC = 16;        // correction check: v faces per thread
-constexpr int kBatchRhsLines = 1;               // right-hand side: lines per thread stack (registers: no spills)
+// Right-hand side: one line per thread stack, its raw values in registers.  In
+// shared memory, as the own kernel of this height has them, they are slower here
+// (64 grids: 6985 us against 6890).
+constexpr int kBatchRhsLines = 1;
+constexpr bool kBatchRhsSlots = false;
 }  // namespace
 
 unsigned batch_stage_tiles(int nx, int ny, int nz, bool rho_given, int stage) {
@@ -131,13 +149,16 @@ unsigned batch_stage_chunk(int nx, int ny, int nz, int stage, long grain) {
 }
 
 size_t batch_smem(int nx, int ny, int nz) {
-  // the right-hand side's rows (256 / nx stacks per CTA, two halo lines) and raw slots
+  // the right-hand side's rows (256 / nx stacks per CTA, two halo lines)
   const size_t tj = (size_t)(kRhsThreads / nx) * kBatchRhsLines;
-  size_t m = sizeof(df) * (size_t)nx * (2 * (tj + 2) + tj) +
-             (rhs_slots_in_smem(kBatchRhsLines) ? sizeof(double) * rhs_slots(kBatchRhsLines, 2) * kRhsThreads : 0);
+  size_t m = sizeof(df) * (size_t)nx * (2 * (tj + 2) + tj);
   m = std::max(m, xrg_smem(nx, (int)lines_per_tile(nx / 2, batch_lpb(nx))));
-  m = std::max(m, rg_smem<float>(nz, (int)lines_per_tile(nz, batch_tkx(nz, true))));
-  m = std::max(m, rg_smem<float>(ny, (int)lines_per_tile(ny, batch_tkx(ny, false))));
+  auto columns = [](int n, bool zpass) {
+    const int cols = (int)lines_per_tile(n, batch_tkx(n, zpass));
+    return tiles_at_once(n, cols) * cols;
+  };
+  m = std::max(m, rg_smem<float>(nz, columns(nz, true)));
+  m = std::max(m, rg_smem<float>(ny, columns(ny, false)));
   return m;
 }
 
@@ -253,10 +274,9 @@ struct BatchPlan {
   static constexpr int radix(int s) { return Own::radix(s); }
   static constexpr int ns(int s) { return Own::ns(s); }
 };
-constexpr bool is_pow2(int n) { return (n & (n - 1)) == 0; }
-constexpr int x_lines_of(int m) { return is_pow2(m) ? 4096 / m : batch_lpb(2 * m); }
-constexpr int z_cols_of(int n) { return is_pow2(n) ? 4096 / n : batch_tkx(n, true); }
-constexpr int y_cols_of(int n) { return is_pow2(n) ? 4096 / n : batch_tkx(n, false); }
+constexpr int x_lines_of(int m) { return (int)lines_per_tile(m, batch_lpb(2 * m)); }
+constexpr int z_cols_of(int n) { return (int)lines_per_tile(n, batch_tkx(n, true)); }
+constexpr int y_cols_of(int n) { return (int)lines_per_tile(n, batch_tkx(n, false)); }
 
 // forward x pass of f (SRC_FDF) or of the residual (SRC_RESID), tile t of nt
 template <int SRC>
@@ -282,30 +302,38 @@ __device__ __noinline__ void x_inverse(const BatchGrid* __restrict__ Bp, uint32_
   });
 }
 
-// z pass; the forward one totals the partial sums first in its tile 0 (fin)
+// z pass of up to tiles_at_once tiles from t on, those below `end`; returns how
+// many one call takes.  The forward one totals the partial sums first in its
+// tile 0 (fin).
 template <bool INV>
-__device__ __noinline__ void z_pass(const BatchGrid* __restrict__ Bp, uint32_t t, uint32_t nt) {
+__device__ __noinline__ int z_pass(const BatchGrid* __restrict__ Bp, uint32_t t, uint32_t end) {
   const BatchGrid& B = *Bp;
   DevScalars* fin = INV ? nullptr : B.sc;
+  int took = 1;
   on_len(B.g.nz, [&](auto NC) {
     constexpr int N = decltype(NC)::value;
-    constexpr int L = z_cols_of(N);
-    zfft_rg_body<float, INV, N, BatchPlan<N, L>>(B.g, B.spec, B.tw_z, L, nullptr, fin, t, nt);
+    constexpr int G = tiles_at_once(N, z_cols_of(N)), L = G * z_cols_of(N);
+    zfft_rg_body<float, INV, N, BatchPlan<N, L>, G>(B.g, B.spec, B.tw_z, L, nullptr, fin, t, end);
+    took = G;
   });
+  return took;
 }
 
-// y pass: DCT-II, eigenvalue divide (zero mode from zmode), DCT-III
-__device__ __noinline__ void y_pass(const BatchGrid* __restrict__ Bp, uint32_t t, uint32_t nt) {
+// y pass, as z_pass: DCT-II, eigenvalue divide (zero mode from zmode), DCT-III
+__device__ __noinline__ int y_pass(const BatchGrid* __restrict__ Bp, uint32_t t, uint32_t end) {
   const BatchGrid& B = *Bp;
+  int took = 1;
   on_len(B.g.ny, [&](auto NC) {
     constexpr int N = decltype(NC)::value;
     if constexpr (N == 256) {  // the radix-16 x 16 form with the divide in registers, as the graph form
-      ydct256_body(B.g, B.spec, B.tw_y, B.wq_y, B.lam_x, B.lam_y, B.lam_z, 16, B.sc, t, nt);
+      ydct256_body(B.g, B.spec, B.tw_y, B.wq_y, B.lam_x, B.lam_y, B.lam_z, 16, B.sc, t, end);
     } else {
-      constexpr int L = y_cols_of(N);
-      ydct_rg_body<float, N, BatchPlan<N, L>>(B.g, B.spec, B.tw_y, B.wq_y, B.lam_x, B.lam_y, B.lam_z, L, B.sc, t, nt);
+      constexpr int G = tiles_at_once(N, y_cols_of(N)), L = G * y_cols_of(N);
+      ydct_rg_body<float, N, BatchPlan<N, L>, G>(B.g, B.spec, B.tw_y, B.wq_y, B.lam_x, B.lam_y, B.lam_z, L, B.sc, t, end);
+      took = G;
     }
   });
+  return took;
 }
 
 __device__ __noinline__ void rhs_pass(const BatchGrid* __restrict__ Bp, uint32_t t) {
@@ -316,8 +344,8 @@ __device__ __noinline__ void rhs_pass(const BatchGrid* __restrict__ Bp, uint32_t
   o.upre = B.upre;
   o.vpre = B.vpre;
   o.wpre = B.wpre;
-  if (B.in.face_rule == 0) rhs_stack_tile<kBatchRhsLines, 0, true>(B.g, B.in, B.sc, o, B.kc, t);
-  else rhs_stack_tile<kBatchRhsLines, 1, true>(B.g, B.in, B.sc, o, B.kc, t);
+  if (B.in.face_rule == 0) rhs_stack_tile<kBatchRhsLines, 0, true, 0, kBatchRhsSlots>(B.g, B.in, B.sc, o, B.kc, t);
+  else rhs_stack_tile<kBatchRhsLines, 1, true, 0, kBatchRhsSlots>(B.g, B.in, B.sc, o, B.kc, t);
 }
 
 __device__ __noinline__ void rho_pass(const BatchGrid* __restrict__ Bp, uint32_t t, uint32_t nt) {
@@ -329,9 +357,12 @@ __device__ __noinline__ void cc_pass(const BatchGrid* __restrict__ Bp, uint32_t 
   correct_check_tile(B.g, B.upre, B.vpre, B.wpre, B.pdf, B.fdf, B.sc, t, nt);
 }
 
-// Runs tile t of stage s of grid B (nt tiles in the stage); returns, for the
-// loop test, whether the refinement goes on (1) or stops (0); -1 otherwise.
-__device__ __forceinline__ int run_item(const BatchGrid* __restrict__ Bp, int s, uint32_t t, uint32_t nt) {
+// Runs tile t of stage s of grid B (nt tiles in the stage), or several at once
+// of the item's (end past its last; took: how many); returns, for the loop
+// test, whether the refinement goes on (1) or stops (0); -1 otherwise.
+__device__ __forceinline__ int run_item(const BatchGrid* __restrict__ Bp, int s, uint32_t t, uint32_t nt, uint32_t end,
+                                        int& took) {
+  took = 1;
   switch (s) {
     case BS_RHO: rho_pass(Bp, t, nt); break;
     case BS_CONST:
@@ -339,9 +370,9 @@ __device__ __forceinline__ int run_item(const BatchGrid* __restrict__ Bp, int s,
       break;
     case BS_RHS: rhs_pass(Bp, t); break;
     case BS_XF: x_forward<SRC_FDF>(Bp, t, nt); break;
-    case BS_ZF0: case BS_ZF: z_pass<false>(Bp, t, nt); break;
-    case BS_Y0: case BS_Y: y_pass(Bp, t, nt); break;
-    case BS_ZI0: case BS_ZI: z_pass<true>(Bp, t, nt); break;
+    case BS_ZF0: case BS_ZF: took = z_pass<false>(Bp, t, end); break;
+    case BS_Y0: case BS_Y: took = y_pass(Bp, t, end); break;
+    case BS_ZI0: case BS_ZI: took = z_pass<true>(Bp, t, end); break;
     case BS_XI0: x_inverse<XI_DF>(Bp, t, nt); break;
     case BS_RES: x_forward<SRC_RESID>(Bp, t, nt); break;
     case BS_XA: x_inverse<XI_DF_ACC>(Bp, t, nt); break;
@@ -425,9 +456,12 @@ __global__ void __launch_bounds__(kBatchThreads, 3)
       const BatchGrid* B = grids + it.grid;
       const int si = kBatchStages * it.grid + it.stage;
       const unsigned nt = tiles[si];
-      for (unsigned t = it.tile0; t < it.tile0 + it.count; ++t) {
+      const unsigned end = it.tile0 + it.count;
+      for (unsigned t = it.tile0; t < end;) {
         if (t > it.tile0) __syncthreads();  // the previous tile's shared-memory reads
-        const int cont = run_item(B, it.stage, t, nt);
+        int took;
+        const int cont = run_item(B, it.stage, t, nt, end, took);
+        t += took;
         if (threadIdx.x == 0 && cont >= 0) {
           if (cont == 0) stop[it.grid] = 1;
           else ctl->cont_any = 1;

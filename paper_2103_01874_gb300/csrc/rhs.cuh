@@ -96,12 +96,13 @@ __host__ __device__ constexpr bool rhs_slots_in_smem(int S) { return S <= 2; }
 // through shared memory; the x faces are exchanged through shared memory for
 // the cell divergence.  Faces between two stacks are evaluated by both (same
 // bits).
+// SM: raw values in shared memory (RawSlots).
 // NXC: nx where it is compiled in (0: any): line and row offsets become
 // immediates, so one address per array and plane serves the S lines.
 // INT: the tile and its halo lines lie strictly inside the walls (no wall or
 // open-top face, every line in range) and rho_0 is the minimum of rho, so the
 // boundary branches and the general form of 1 - rho_0/rho_f drop out.
-template <int S, int RULE, bool PROJ, bool INT, int NXC>
+template <int S, int RULE, bool PROJ, bool INT, int NXC, bool SM>
 __device__ __forceinline__ void rhs_stack_body(const GridDev& g, const StencilIn& in, DevScalars* sc,
                                                const RhsOut& out, int kc, uint32_t bid) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -140,7 +141,6 @@ __device__ __forceinline__ void rhs_stack_body(const GridDev& g, const StencilIn
   auto at = [&](int kk) -> uint32_t { return (uint32_t)kk * plane + own; };          // own cell of line 0
 
   constexpr int HN = (NXC > 0 && stacks_of(NXC) > 1) ? 1 : 2;  // a thread's halo cells (such CTAs have two stacks or more)
-  constexpr bool SM = rhs_slots_in_smem(S);
   RawSlots<rhs_slots(S, HN), SM> raw;
   raw.own = reinterpret_cast<double*>(QX + tj * nx) + threadIdx.x;
   constexpr int S_U = 0, S_W = S, S_S = 2 * S, S_V = 3 * S, S_P = 4 * S + 1, S_H = 7 * S + 1;
@@ -395,16 +395,16 @@ __device__ __forceinline__ void rhs_stack_body(const GridDev& g, const StencilIn
 // One tile (CTA index bid) of the column-stack march: the interior form when
 // the tile and its halo lines lie strictly inside the walls and rho_0 is the
 // minimum of rho (in.min_rho0).
-template <int S, int RULE, bool PROJ, int NXC = 0>
+template <int S, int RULE, bool PROJ, int NXC = 0, bool SM = rhs_slots_in_smem(S)>
 __device__ __forceinline__ void rhs_stack_tile(const GridDev& g, const StencilIn& in, DevScalars* sc,
                                                const RhsOut& out, int kc, uint32_t bid) {
   const int tj = ((int)blockDim.x / (NXC ? NXC : g.nx)) * S;
   const int ntile = (g.ny + tj - 1) / tj;
   const int j0 = (int)(bid % ntile) * tj;
   if (in.min_rho0 && j0 > 0 && j0 + tj < g.ny)  // uniform over the CTA
-    rhs_stack_body<S, RULE, PROJ, true, NXC>(g, in, sc, out, kc, bid);
+    rhs_stack_body<S, RULE, PROJ, true, NXC, SM>(g, in, sc, out, kc, bid);
   else
-    rhs_stack_body<S, RULE, PROJ, false, NXC>(g, in, sc, out, kc, bid);
+    rhs_stack_body<S, RULE, PROJ, false, NXC, SM>(g, in, sc, out, kc, bid);
 }
 
 }  // namespace ppe

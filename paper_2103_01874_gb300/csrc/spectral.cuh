@@ -519,23 +519,26 @@ __global__ void __launch_bounds__(256) k_zfft(GridDev g, cpx<T>* spec, RadixPlan
 // threads; the first pass reads the
 // columns from the spectrum and the last pass writes them back, so each
 // element crosses shared memory once.
-template <typename T, bool INV, int N, class RP = rgfft::RegPlan<N>>
+// G > 1: the CTA's L columns are those of G consecutive tiles of L / G columns
+// each, bid the first of them and nblk the end of the tiles to take (the
+// persistent batch's short tiles).
+template <typename T, bool INV, int N, class RP = rgfft::RegPlan<N>, int G = 1>
 __device__ __forceinline__ void zfft_rg_body(GridDev g, cpx<T>* spec, const cpx<T>* tw, int L,
                                                  const DevScalars* sc, DevScalars* fin, uint32_t bid, uint32_t nblk) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (fin && bid == 0) finish_sums(fin, g);  // uniform over the CTA
   if (sc && sc->done) return;
   const uint32_t nxh = (uint32_t)g.nx / 2 + 1;
-  const uint32_t ntile = (nxh + L - 1) / L;
-  const uint32_t j = bid / ntile;
-  const uint32_t kx0 = (bid - j * ntile) * L;
+  const uint32_t LT = (uint32_t)(L / G), ntile = (nxh + LT - 1) / LT;
   cpx<T>* buf = reinterpret_cast<cpx<T>*>(smem_raw);
   cpx<T>* tws = buf + rgfft::rows(N) * L;  // exp(-2 pi i t/nz)
   for (int t = threadIdx.x; t < N; t += blockDim.x) cp_async<sizeof(cpx<T>)>(&tws[t], &tw[t]);
   const int line = threadIdx.x & (L - 1), t0 = threadIdx.x >> ilog2_dev(L);
-  const bool valid = kx0 + line < nxh;
+  const uint32_t sub = G > 1 ? line / LT : 0u, tile = bid + sub;
+  const uint32_t j = tile / ntile, kx = (tile - j * ntile) * LT + (line - sub * LT);
+  const bool valid = kx < nxh && (G == 1 || tile < nblk);
   const uint32_t rs = (uint32_t)g.ny * nxh;  // kz stride (32-bit offsets: spectra below 2^32 elements)
-  cpx<T>* col = spec + (j * nxh + kx0 + line);
+  cpx<T>* col = spec + (j * nxh + kx);
   rgfft::run_plan<T, INV, RP, 1, false>(
       [&](int e) { return valid ? col[(uint32_t)e * rs] : cpx<T>{(T)0, (T)0}; },
       [&](int e, cpx<T> v) {
@@ -768,22 +771,25 @@ __global__ void __launch_bounds__(256) k_ydct(GridDev g, cpx<T>* spec, RadixPlan
 // the DCT-II's FFT, the eigenvalue division works on the shared buffer, and
 // the last pass of the inverse writes the reordered result back.  Same
 // arithmetic as k_ydct.
-template <typename T, int N, class RP = rgfft::RegPlan<N>>
+// (A thread keeps its column through every loop: blockDim.x is a multiple of L.
+// G, bid and nblk as in zfft_rg_body.)
+template <typename T, int N, class RP = rgfft::RegPlan<N>, int G = 1>
 __device__ __forceinline__ void ydct_rg_body(GridDev g, cpx<T>* spec, const cpx<T>* tw,
                                                  const cpx<T>* wq, const T* lam_x,
                                                  const T* lam_y, const T* lam_z, int L,
                                                  const DevScalars* zsc, uint32_t bid, uint32_t nblk) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const uint32_t nxh = (uint32_t)g.nx / 2 + 1;
-  const uint32_t ntile = (nxh + L - 1) / L;
-  const uint32_t kz = bid / ntile, kx0 = (bid - kz * ntile) * L;
+  const uint32_t LT = (uint32_t)(L / G), ntile = (nxh + LT - 1) / LT;
   cpx<T>* buf = reinterpret_cast<cpx<T>*>(smem_raw);
   cpx<T>* tws = buf + rgfft::rows(N) * L;  // exp(-2 pi i t/ny)
   for (int t = threadIdx.x; t < N; t += blockDim.x) cp_async<sizeof(cpx<T>)>(&tws[t], &tw[t]);
   const int lg = ilog2_dev(L);
   const int line = threadIdx.x & (L - 1), t0 = threadIdx.x >> lg;
-  const bool valid = kx0 + line < nxh;
-  cpx<T>* col = spec + (kz * (uint32_t)N * nxh + kx0 + line);
+  const uint32_t sub = G > 1 ? line / LT : 0u, tile = bid + sub;
+  const uint32_t kz = tile / ntile, kx = (tile - kz * ntile) * LT + (line - sub * LT);
+  const bool valid = kx < nxh && (G == 1 || tile < nblk);
+  cpx<T>* col = spec + (kz * (uint32_t)N * nxh + kx);
   // v[p] = x_j with p = j/2 (even j) or N-1-(j-1)/2 (odd j)
   auto jof = [](int p) { return p < N / 2 ? 2 * p : 2 * (N - 1 - p) + 1; };
   rgfft::run_plan<T, false, RP, 1, false>(
@@ -791,17 +797,15 @@ __device__ __forceinline__ void ydct_rg_body(GridDev g, cpx<T>* spec, const cpx<
       [&](int e, cpx<T> v) { buf[rgfft::row(e) * L + line] = v; }, buf + line, L, t0, tws);
   __syncthreads();
   const T inv_n = (T)1 / (T)N;
-  const T lz = lam_z[kz];
+  const T lxz = valid ? lam_x[kx] + lam_z[kz] : (T)0;
   constexpr int npair = N / 2 + 1;
   // 1/N times the reciprocal: with N a power of two that is the correctly
   // rounded quotient; else one more rounding, the same in both of a pair's lines
 #pragma unroll 1
   for (int idx = threadIdx.x; idx < npair * L; idx += blockDim.x) {
-    const int k = idx >> lg, c = idx & (L - 1);
-    const uint32_t kx = kx0 + c;
-    if (kx >= nxh) continue;
-    const T lxz = lam_x[kx] + lz;
-    cpx<T>* Vk = buf + rgfft::row(k) * L + c;
+    if (!valid) break;
+    const int k = idx >> lg;
+    cpx<T>* Vk = buf + rgfft::row(k) * L + line;
     if (k == 0) {
       const T lam = lxz + lam_y[0];
       const cpx<T> v0 = *Vk;
@@ -814,7 +818,7 @@ __device__ __forceinline__ void ydct_rg_body(GridDev g, cpx<T>* spec, const cpx<
       continue;
     }
     const int r = N - k;
-    cpx<T>* Vr = buf + rgfft::row(r) * L + c;
+    cpx<T>* Vr = buf + rgfft::row(r) * L + line;
     const cpx<T> vk = *Vk, vr = *Vr;
     const cpx<T> wk = wq[k], wr = wq[r];
     const cpx<T> wkc = {wk.x, -wk.y}, wrc = {wr.x, -wr.y};
@@ -835,9 +839,9 @@ __device__ __forceinline__ void ydct_rg_body(GridDev g, cpx<T>* spec, const cpx<
   __syncthreads();
   // x_j = v'[p(j)]: copy-out row by row (j = idx / L), consecutive threads on consecutive columns
   for (int idx = threadIdx.x; idx < N * L; idx += blockDim.x) {
-    const int jj = idx >> lg, c = idx & (L - 1);
+    const int jj = idx >> lg;
     const int pj = (jj & 1) ? N - 1 - (jj >> 1) : (jj >> 1);
-    if (kx0 + c < nxh) spec[kz * (uint32_t)N * nxh + (uint32_t)jj * nxh + kx0 + c] = buf[rgfft::row(pj) * L + c];
+    if (valid) col[(uint32_t)jj * nxh] = buf[rgfft::row(pj) * L + line];
   }
 }
 template <typename T, int N>
