@@ -379,7 +379,12 @@ int rhs_max_lines(int nx) {
 namespace {
 // Calls f(kernel) with the column-stack instance for (S, rule, proj, nx).
 // The projection's default S = 2 has instances with nx compiled in for the
-// usual widths (their CTAs are whole stacks: threads = stacks * nx).
+// widths 2^a and 3 2^a that are whole warps, up to 384: their CTAs are whole
+// stacks (threads = stacks * nx) and offsets are immediates, without and with us
+// (min rho_0, cubes; 384 x 256 x 128): 32 11.6 -> 9.7, 64 16 -> 14, 96 36 -> 27, 128
+// 59 -> 49, 192 170 -> 136, 256 371 -> 304, 384 291 -> 243.  An instance would
+// buy 4 % at 144 (93 -> 89) and 2 % at 512 (349 -> 341), 2 us at 48 (12.6 -> 10.7),
+// for two kernels of build each; ppe_rhs and the other heights take any nx.
 template <int S, int RULE, bool PROJ, class F>
 void stack_instance(int nx, int threads, F&& f) {
   if constexpr (S == 2 && PROJ) {

@@ -394,7 +394,11 @@ __device__ __forceinline__ void rhs_stack_body(const GridDev& g, const StencilIn
 
 // One tile (CTA index bid) of the column-stack march: the interior form when
 // the tile and its halo lines lie strictly inside the walls and rho_0 is the
-// minimum of rho (in.min_rho0).
+// minimum of rho (in.min_rho0).  With a caller's rho_0 every tile takes the
+// boundary form (256^3: 360 us against 304; the form with a flux per face took
+// 375 with either).  A third body in the same kernel, interior with the general
+// difference, brings that to 319 but costs the usual case registers: 384 x 256 x
+// 128 243 -> 256 us, 144^3 93 -> 97, and 128^3 with a caller's rho_0 55 -> 58.
 template <int S, int RULE, bool PROJ, int NXC = 0, bool SM = rhs_slots_in_smem(S)>
 __device__ __forceinline__ void rhs_stack_tile(const GridDev& g, const StencilIn& in, DevScalars* sc,
                                                const RhsOut& out, int kc, uint32_t bid) {
