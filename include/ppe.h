@@ -382,7 +382,12 @@ void ppe_destroy(ppe_plan_t plan);
  * is outside its range, a schedule is not available for the plan, or a pass
  * would need more than 227 KB of shared memory per CTA.  Synchronises the
  * plan's stream (captured refinement graphs are rebuilt with the new
- * schedule). */
+ * schedule).  It gives every field; ppe_set_tuning_fields gives those named in
+ * `given` (bit i: the struct's i-th field, PPE_TUNE_*) and keeps the plan's value
+ * of the others.  A plan's rhs_planes is chosen so that its grid alone fills the
+ * GPU until a call gives it; in the graph form of a batch, whose grids fill the
+ * GPU together, a plan's own choice is raised to min(8, nz) and a given value is
+ * taken as it is. */
 enum { PPE_SPECTRAL_LEGACY = 0, PPE_SPECTRAL_FUSED = 1, PPE_SPECTRAL_PENCIL = 2 };
 enum { PPE_Y_COSINE = 0, PPE_Y_TRIDIAGONAL = 1 };
 typedef struct {
@@ -390,6 +395,11 @@ typedef struct {
 } ppe_tuning;
 ppe_status ppe_get_tuning(ppe_plan_t plan, ppe_tuning* out);
 ppe_status ppe_set_tuning(ppe_plan_t plan, const ppe_tuning* tuning);
+enum {
+    PPE_TUNE_RHS_LINES = 1, PPE_TUNE_RHS_PLANES = 2, PPE_TUNE_X_LINES = 4, PPE_TUNE_Z_COLS = 8,
+    PPE_TUNE_Y_COLS = 16, PPE_TUNE_SPECTRAL = 32, PPE_TUNE_Y_SOLVE = 64, PPE_TUNE_ALL = 127
+};
+ppe_status ppe_set_tuning_fields(ppe_plan_t plan, const ppe_tuning* tuning, unsigned given);
 
 /* Per-kernel timing.  While enabled, every kernel the plan launches is
  * bracketed by two CUDA events on the plan's stream.  ppe_profile_read

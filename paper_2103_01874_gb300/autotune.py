@@ -79,7 +79,8 @@ def apply_cached(plan: "ppe.Plan", path: str = DEFAULT_CACHE, gpu: str | None = 
     if not entry:
         return False
     try:
-        plan.set_tuning(**entry["tuning"])
+        # (what the search left out stays the plan's own choice)
+        plan.set_tuning(**{k: v for k, v in entry["tuning"].items() if k in entry.get("kernel_us", entry["tuning"])})
     except ppe.PPEError:
         return False
     return True
@@ -106,15 +107,13 @@ def autotune(plan: "ppe.Plan", run, reps: int = 3, path: str | None = DEFAULT_CA
     Returns {"tuning": best shapes, "kernel_us": time of each tuned kernel}."""
     search = SEARCH if search is None else search
     run(1)  # warm-up and first-use costs
-    best = plan.get_tuning()
+    best = {}  # the searched fields alone are given to the plan
     times = {}
     for field, (kernel, values) in search.items():
         scores = []
         for v in values:
-            trial = dict(best)
-            trial[field] = v
             try:
-                plan.set_tuning(**trial)
+                plan.set_tuning(**dict(best, **{field: v}))
             except ppe.PPEError:
                 continue  # out of range, too much shared memory, or a schedule this plan lacks
             if kernel == STEP:
@@ -125,7 +124,7 @@ def autotune(plan: "ppe.Plan", run, reps: int = 3, path: str | None = DEFAULT_CA
             best[field] = v
             times[field] = {"kernel": kernel, "us": t, "tried": {str(b): a for a, b in scores}}
         plan.set_tuning(**best)
-    result = {"tuning": best, "kernel_us": times}
+    result = {"tuning": plan.get_tuning(), "kernel_us": times}
     if path:
         cache = load_cache(path)
         cache[cache_key(plan)] = result

@@ -42,6 +42,7 @@ struct ppe_plan_s {
   int* line_len;
   double a_y;         // 1/dy^2
   int tj, kc;         // right-hand-side kernel: lines per tile, planes per chunk
+  bool kc_given;      // kc was given by a ppe_set_tuning call
   df* fdf;            // FP32_REFINE: right-hand side as pairs, kept for the residual
   df* pdf;            // FP32_REFINE: pressure as pairs during the refinement
   float* p32;         // FP32_REFINE, register-staged x passes, (nx/2) nz a power of two, max_sweeps >= 1:
@@ -1025,8 +1026,20 @@ ppe_status ppe_get_tuning(ppe_plan_t P, ppe_tuning* t) {
   return PPE_OK;
 }
 
-ppe_status ppe_set_tuning(ppe_plan_t P, const ppe_tuning* t) {
-  if (!P || !t) return PPE_ERR_INVALID_ARG;
+ppe_status ppe_set_tuning(ppe_plan_t P, const ppe_tuning* t) { return ppe_set_tuning_fields(P, t, PPE_TUNE_ALL); }
+
+ppe_status ppe_set_tuning_fields(ppe_plan_t P, const ppe_tuning* in, unsigned given) {
+  if (!P || !in || (given & ~(unsigned)PPE_TUNE_ALL)) return PPE_ERR_INVALID_ARG;
+  ppe_tuning all, prev;
+  ppe_get_tuning(P, &prev);
+  all.rhs_lines = given & PPE_TUNE_RHS_LINES ? in->rhs_lines : prev.rhs_lines;
+  all.rhs_planes = given & PPE_TUNE_RHS_PLANES ? in->rhs_planes : prev.rhs_planes;
+  all.x_lines = given & PPE_TUNE_X_LINES ? in->x_lines : prev.x_lines;
+  all.z_cols = given & PPE_TUNE_Z_COLS ? in->z_cols : prev.z_cols;
+  all.y_cols = given & PPE_TUNE_Y_COLS ? in->y_cols : prev.y_cols;
+  all.spectral = given & PPE_TUNE_SPECTRAL ? in->spectral : prev.spectral;
+  all.y_solve = given & PPE_TUNE_Y_SOLVE ? in->y_solve : prev.y_solve;
+  const ppe_tuning* const t = &all;
   auto pow2 = [](int v, int lo, int hi) { return v >= lo && v <= hi && (v & (v - 1)) == 0; };
   const size_t lim = 227 * 1024;
   const int nx = P->g.nx, ny = P->g.ny, nz = P->g.nz;
@@ -1052,8 +1065,6 @@ ppe_status ppe_set_tuning(ppe_plan_t P, const ppe_tuning* t) {
     cudaGraphExecDestroy(P->pcg_exec);
     P->pcg_exec = nullptr;
   }
-  ppe_tuning prev;
-  ppe_get_tuning(P, &prev);
   auto apply = [&](const ppe_tuning& u) {
     P->tj = u.rhs_lines;
     P->kc = u.rhs_planes;
@@ -1066,6 +1077,7 @@ ppe_status ppe_set_tuning(ppe_plan_t P, const ppe_tuning* t) {
   };
   const ppe_status s = apply(*t);
   if (s != PPE_OK) apply(prev);  // the plan keeps its previous shapes and graphs
+  else if (given & PPE_TUNE_RHS_PLANES) P->kc_given = true;
   return s;
 }
 
@@ -1488,8 +1500,8 @@ ppe_status batch_graph(ppe_batch_t B, int n, const ppe_plan_t* plans, const ppe_
     P->stream = bs[branch[i]];
     // the branches fill the GPU together: a right-hand side's planes per CTA,
     // chosen short so that a small grid alone fills it, march at least eight
-    // here (64 grids: 3994 -> 3910 us), unless they were set
-    if (kc == rhs_planes(P->g.nx, P->g.ny, P->g.nz)) P->kc = std::max(kc, std::min(8, P->g.nz));
+    // here (64 grids: 3994 -> 3901 us), unless a ppe_set_tuning call gave them
+    if (!P->kc_given) P->kc = std::max(kc, std::min(8, P->g.nz));
     st = ppe_project(P, &fields[i]);
     P->kc = kc;
     P->stream = saved;

@@ -116,6 +116,7 @@ SIGNATURES = {
     "ppe_batch_schedule": (ctypes.c_longlong, [c_int, POINTER(c_int), POINTER(c_int), c_int, c_int, c_int, c_int,
                                                POINTER(c_int), ctypes.c_longlong, POINTER(c_int), POINTER(c_int)]),
     "ppe_set_tuning": (c_int, [c_void_p, POINTER(Tuning)]),
+    "ppe_set_tuning_fields": (c_int, [c_void_p, POINTER(Tuning), ctypes.c_uint]),
     "ppe_profile_read": (c_int, [c_void_p, POINTER(KernelTime), c_int]),
     "ppe_project_unsplit": (c_int, [c_void_p, POINTER(FieldsC), c_double, c_int]),
     "ppe_unsplit_info": (c_int, [c_void_p, POINTER(c_int), POINTER(c_double)]),
@@ -401,11 +402,10 @@ class Plan:
         return t.as_dict()
 
     def set_tuning(self, **kw):
-        """Change launch shapes (ppe_set_tuning); unspecified fields keep their value."""
-        cur = self.get_tuning()
-        cur.update(kw)
-        t = Tuning(**cur)
-        _check(lib().ppe_set_tuning(self._h, ctypes.byref(t)), "ppe_set_tuning")
+        """Change launch shapes (ppe_set_tuning_fields); unspecified fields keep their value."""
+        t = Tuning(**kw)
+        given = sum(1 << i for i, (k, _) in enumerate(Tuning._fields_) if k in kw)
+        _check(lib().ppe_set_tuning_fields(self._h, ctypes.byref(t), given), "ppe_set_tuning")
 
     def profile(self, enable: bool):
         _check(lib().ppe_profile(self._h, 1 if enable else 0), "ppe_profile")
