@@ -12,17 +12,21 @@ ppe_set_tuning exposes two kinds of choices:
     so each is scored by that kernel alone.
 `autotune` searches them coordinate by coordinate on the caller's own fields
 (the schedule first, since it decides which kernels the tile sizes drive),
-applies the best and remembers it in a JSON cache keyed by grid, precision,
-face rule and GPU name, so that later plans of the same size class start from
-it (`apply_cached`).
+applies the best and remembers it in a JSON cache keyed by the kernel sources,
+grid, precision, face rule, top boundary and GPU name, so that later plans of
+the same size class start from it (`apply_cached`); an entry tuned on other
+sources, whose defaults and kernels may differ, is not found.  The value that a
+plan has is always among those tried.
 """
 from __future__ import annotations
 
+import functools
+import hashlib
 import json
 import os
 import threading
 
-from . import ppe
+from . import build, ppe
 
 DEFAULT_CACHE = os.path.join(os.path.expanduser("~"), ".cache", "ppe_gb300", "tuning.json")
 
@@ -34,7 +38,7 @@ SEARCH = {
     "spectral": (STEP, (0, 1, 2)),
     "y_solve": (STEP, (1, 0)),
     "rhs_lines": ("k_rhs_march", (1, 2, 4, 8)),
-    "rhs_planes": ("k_rhs_march", (4, 8, 16, 32)),
+    "rhs_planes": ("k_rhs_march", (1, 2, 3, 4, 6, 8, 10, 12, 16, 32)),  # (a plan's own choice: 1 .. 12)
     "x_lines": ("k_xinv", (4, 8, 16, 32, 64)),
     "z_cols": ("k_zfft_fwd", (2, 4, 8, 16)),
     "y_cols": ("k_ysolve", (2, 4, 8, 16, 32)),
@@ -51,9 +55,19 @@ def _gpu_name() -> str:
         return "unknown"
 
 
+@functools.lru_cache(maxsize=1)
+def kernels_version() -> str:
+    """Short hash of the library's sources."""
+    h = hashlib.sha256()
+    for path in sorted(build._deps()):
+        with open(path, "rb") as fh:
+            h.update(os.path.basename(path).encode() + b"\0" + fh.read())
+    return h.hexdigest()[:12]
+
+
 def cache_key(plan: "ppe.Plan", gpu: str | None = None) -> str:
-    return (f"{plan.nx}x{plan.ny}x{plan.nz}|prec{plan.precision}|face{plan.opts.face_rule}|"
-            f"{gpu if gpu is not None else _gpu_name()}")
+    return (f"{kernels_version()}|{plan.nx}x{plan.ny}x{plan.nz}|prec{plan.precision}|face{plan.opts.face_rule}|"
+            f"top{getattr(plan.opts, 'bc_top', ppe.BC_WALL)}|{gpu if gpu is not None else _gpu_name()}")
 
 
 def load_cache(path: str = DEFAULT_CACHE) -> dict:
@@ -111,7 +125,8 @@ def autotune(plan: "ppe.Plan", run, reps: int = 3, path: str | None = DEFAULT_CA
     times = {}
     for field, (kernel, values) in search.items():
         scores = []
-        for v in values:
+        own = plan.get_tuning()[field]
+        for v in (*values, *(() if own in values else (own,))):
             try:
                 plan.set_tuning(**dict(best, **{field: v}))
             except ppe.PPEError:
