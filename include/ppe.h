@@ -112,7 +112,8 @@ typedef struct {
                          * always drops the mean of f (reported in
                          * ppe_info.f_mean_removed); with compat_tol > 0, ppe_get_info
                          * and ppe_project_host also return PPE_ERR_INCOMPATIBLE_RHS
-                         * when |mean(f)| > compat_tol * ||f||_inf.  0: no check.  The
+                         * when |mean(f)| > compat_tol * ||f||_inf (plus what a pair
+                         * cannot hold of S or f, below 2^-126).  0: no check.  The
                          * paper has no such check; it follows from the divergence
                          * theorem on the periodic/wall box of Sec. 5. */
     ppe_bc bc_top;      /* top boundary in y (PPE_BC_WALL when opt is NULL) */

@@ -18,8 +18,9 @@
 //
 // Representation: value = hi + lo, |lo| <= ulp(hi)/2 after normalisation.
 // Relative precision ~2^-48 (3.6e-15).  Range: magnitudes in [2^-74, 2^127];
-// below that the low part thins out (denormal) and magnitudes under 2^-126
-// are flushed to a few 1e-45, larger ones are out of scope.
+// below that the low part thins out (denormal), values in [2^-127, 2^-126) lose
+// their leading bit and smaller ones become a few 1e-45 (both with an absolute
+// error of at most 2^-127); larger ones are out of scope.
 //
 // d2df(x): hi = x truncated to 24 significant bits (exponent rebias and
 // mantissa shift on the bit pattern), lo = the remaining 29 mantissa bits as an
@@ -205,6 +206,8 @@ PPE_HD df df_recipz(df a) {
   return {y0, y0 * e};
 }
 
+constexpr double kPairTiny = 0x1p-126;
+
 // max(a + b, 0) on signed integers (one instruction on the device)
 PPE_HD int addmax0(int a, int b) {
 #ifdef __CUDA_ARCH__
@@ -223,7 +226,7 @@ PPE_HD int addmax0(int a, int b) {
 // field).  Nine operations instead of the twelve of a form that tested the
 // range and selected zeros (they are a quarter of the right-hand side's
 // instructions); zeros keep their sign and a zero low part.
-PPE_HD df d2df(double x) {
+PPE_HD df d2df(double x) {  // (kPairTiny bounds the absolute error of a tiny x)
   const uint64_t b = d_bits(x);
   const uint32_t hw = (uint32_t)(b >> 32), lw = (uint32_t)b;
   const uint32_t m = (uint32_t)addmax0((int)(hw & 0x7FFFFFFFu), -(896 << 20));

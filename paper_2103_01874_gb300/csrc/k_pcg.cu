@@ -72,10 +72,13 @@ __global__ void __launch_bounds__(256) k_vc_setup(GridDev g, const double* __res
     az[c] = face_coef<RULE>(d2df(__ldg(rho + zm)), rc, C.iz2);
     ay[c] = (q.j == 0) ? df{0.0f, 0.0f} : face_coef<RULE>(d2df(__ldg(rho + c - nx)), rc, C.iy2);  // wall: no flux
     const uint32_t cv = (q.k * (ny + 1) + q.j) * nx + q.i;  // v face below the cell
-    const df du = df_addz(df_addz(df_mulz(df_sub(d2df(__ldg(u + xp)), d2df(__ldg(u + c))), C.idx),
-                                  df_mulz(df_sub(d2df(__ldg(v + cv + nx)), d2df(__ldg(v + cv))), C.idy)),
-                          df_mulz(df_sub(d2df(__ldg(w + zp)), d2df(__ldg(w + c))), C.idz));
-    const df gv = df_norm(df_mulz(df_subz(d2df(__ldg(S + c)), du), C.idt));
+    // g of values below 2^-74 is zero: the dot products of the iteration square
+    // it in FP32's range, where 1e-21 is lost
+    auto val = [](const double* a) { return fabs(__ldg(a)) < 0x1p-74 ? df{0.0f, 0.0f} : d2df(__ldg(a)); };
+    const df du = df_addz(df_addz(df_mulz(df_sub(val(u + xp), val(u + c)), C.idx),
+                                  df_mulz(df_sub(val(v + cv + nx), val(v + cv)), C.idy)),
+                          df_mulz(df_sub(val(w + zp), val(w + c)), C.idz));
+    const df gv = df_norm(df_mulz(df_subz(val(S + c), du), C.idt));
     r[c] = gv;
     gsum = df_addz(gsum, gv);
     gmax = fmaxf(gmax, fabsf(gv.hi));

@@ -1711,8 +1711,11 @@ ppe_status info_from(ppe_plan_t P, const DevScalars& h, ppe_info* info) {
     if (h.f_ran && !P->gd.top_open) info->s_mean = info->wall_flux_mean - info->f_mean_removed / df2d(h.K.c);
   }
   // the Neumann problem needs mean(f) = 0; what the solve drops, relative to ||f||
-  // (an open top has no compatibility condition)
-  if (h.f_ran && P->opt.compat_tol > 0 && !P->gd.top_open) incompatible = fabs(h.f_sum / n) > P->opt.compat_tol * fmax;
+  // (an open top has no compatibility condition), beyond what the pairs resolve:
+  // an S (or a caller's f) below kPairTiny has no mean there
+  const double unseen = kPairTiny * (h.rhs_ran ? std::max(1.0, df2d(h.K.c)) : 1.0);
+  if (h.f_ran && P->opt.compat_tol > 0 && !P->gd.top_open)
+    incompatible = fabs(h.f_sum / n) > P->opt.compat_tol * fmax + unseen;
   if (P->fp32) {
     // max_sweeps = 0 applies no correction; the device test that follows the
     // fused correction-and-residual kernel counts that pass as one sweep
