@@ -879,8 +879,8 @@ ppe_status ppe_plan(ppe_plan_t* out, const ppe_grid* g, const ppe_options* opt, 
   P->rp_z = radix_plan(g->nz, maxr);
   P->lpb = choose_lpb(g->nx);
   // the FP64 form's x passes (256-thread CTAs whatever the lines): fewer lines
-  // where the grid would leave SMs without a CTA (64^3: 64 lines, 64 CTAs, 57.5 us
-  // a projection; 16 lines, 256 CTAs, 52.0)
+  // where the grid would leave SMs without a CTA (64^3: 64 lines, 64 CTAs, 58.5 us
+  // a projection; 16 lines, 256 CTAs, 53.9)
   if (!P->fp32)
     while (P->lpb > 16 && (long)g->ny * g->nz / P->lpb < 228) P->lpb /= 2;
   P->tkx = choose_tkx(g->nz, P->fp32, true);

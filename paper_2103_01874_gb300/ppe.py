@@ -32,7 +32,7 @@ SPECTRAL_PENCIL = 2  # three bulk-copy-staged persistent passes, spectrum [kx][k
 Y_COSINE = 0       # DCT-II, eigenvalue divide, DCT-III through FFTs
 Y_TRIDIAGONAL = 1  # Thomas elimination as two affine scans (FP32 with walls, ny <= 512)
 # forms of a batch (ppe_batch_options.form)
-BATCH_AUTO = 0        # persistent where every plan qualifies, else graph
+BATCH_AUTO = 0        # the library's choice: graph, the faster on every batch measured
 BATCH_GRAPH = 1       # graph branches, one per projection
 BATCH_PERSISTENT = 2  # one persistent kernel over a device work queue
 
