@@ -320,14 +320,16 @@ __global__ void __launch_bounds__(BT, BT == 256 ? (S <= 2 ? 3 : (S == 4 ? 2 : 1)
 namespace {
 // Stacks of a launch: those that fill its grid best, within the block bound of
 // the instance of this nx (two at least where it gives a thread one halo cell).
+// Eight lines a thread: 256 threads at most, whose registers and raw slots
+// (129 KB) an SM holds.
 int launch_stacks(int nx, int ny, int S) {
+  if (S == 8) return stacks_of(nx, ny, S, 1, 256);
   const int s0 = stacks_of(nx);
   return stacks_of(nx, ny, S, s0 > 1 ? 2 : 1, stack_bound(stack_threads(nx, s0)));
 }
 size_t stack_smem(int nx, int stacks, int S) {
   const size_t tj = (size_t)stacks * S, nl = tj + 2;
-  return sizeof(df) * (2 * nl * nx + tj * nx) +
-         (rhs_slots_in_smem(S) ? sizeof(double) * rhs_slots(S, 2) * stack_threads(nx, stacks) : 0);
+  return sizeof(df) * (2 * nl * nx + tj * nx) + sizeof(double) * rhs_slots(S, 2) * stack_threads(nx, stacks);
 }
 }  // namespace
 
@@ -378,28 +380,32 @@ int rhs_max_lines(int nx) {
 
 namespace {
 // Calls f(kernel) with the column-stack instance for (S, rule, proj, nx).
-// The projection's default S = 2 has instances with nx compiled in for the
-// widths 2^a and 3 2^a that are whole warps, up to 384: their CTAs are whole
-// stacks (threads = stacks * nx) and offsets are immediates, without and with us
-// (min rho_0, cubes; 384 x 256 x 128): 32 11.6 -> 9.7, 64 16 -> 14, 96 36 -> 27, 128
-// 59 -> 49, 192 170 -> 136, 256 371 -> 304, 384 291 -> 243.  An instance would
-// buy 4 % at 144 (93 -> 89) and 2 % at 512 (349 -> 341), 2 us at 48 (12.6 -> 10.7),
-// for two kernels of build each; ppe_rhs and the other heights take any nx.
+// The default S = 2 has instances with nx compiled in for the widths 2^a and
+// 3 2^a that are whole warps, up to 384: their CTAs are whole stacks (threads =
+// stacks * nx) and offsets are immediates.  Without and with them (projection,
+// min rho_0, cubes; 384 x 256 x 128): 32 11.6 -> 9.7 us, 64 16 -> 14, 96 36 -> 27,
+// 128 59 -> 49, 192 170 -> 136, 256 371 -> 304, 384 291 -> 243; ppe_rhs: 128
+// 55 -> 45, 192 164 -> 131, 256 364 -> 305 (the form with a flux per face took
+// 349).  An instance would buy 4 % at 144 (93 -> 89), 2 % at 512 (349 -> 341) and
+// 2 us at 48 (12.6 -> 10.7), for four kernels of build each.  The other heights
+// take any nx.
 template <int S, int RULE, bool PROJ, class F>
 void stack_instance(int nx, int threads, F&& f) {
-  if constexpr (S == 2 && PROJ) {
+  if constexpr (S == 2) {
 #define PPE_NX(N) \
-    case N: return f(k_rhs_stack<2, RULE, true, stack_bound(stack_threads(N, stacks_of(N))), N>);
+    case N: return f(k_rhs_stack<2, RULE, PROJ, stack_bound(stack_threads(N, stacks_of(N))), N>);
     switch (nx) {
       PPE_NX(32) PPE_NX(64) PPE_NX(96) PPE_NX(128) PPE_NX(192) PPE_NX(256) PPE_NX(384)
       default: break;
     }
 #undef PPE_NX
   }
-  if (threads <= 256) return f(k_rhs_stack<S, RULE, PROJ, 256, 0>);
-  if constexpr (S <= 2)
-    if (threads <= 384) return f(k_rhs_stack<S, RULE, PROJ, 384, 0>);
-  f(k_rhs_stack<S, RULE, PROJ, 512, 0>);
+  if constexpr (S < 8) {
+    if constexpr (S <= 2)
+      if (threads > 256 && threads <= 384) return f(k_rhs_stack<S, RULE, PROJ, 384, 0>);
+    if (threads > 256) return f(k_rhs_stack<S, RULE, PROJ, 512, 0>);
+  }
+  f(k_rhs_stack<S, RULE, PROJ, 256, 0>);
 }
 
 template <int S, class F>

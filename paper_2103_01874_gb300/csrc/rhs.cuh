@@ -50,12 +50,13 @@ struct RhsOut {
 };
 
 // Raw input values of a thread, fetched a phase or more ahead of their use.
-// Up to two lines per thread they wait in shared memory (8-byte cp.async into
-// slots of the thread's own, so that no barrier is needed to reuse one): kept
-// in registers they left room for neither the halo's nor a second plane's
-// loads at 80 registers a thread, and load latency (long scoreboard 3.7 of 9.5
-// cycles per instruction) held the march at 55 % issue.  Taller stacks keep
-// registers: their slots would not fit the shared memory.
+// SMEM: they wait in shared memory (8-byte cp.async into slots of the thread's
+// own, so that no barrier is needed to reuse one): kept in registers they left
+// room for neither the halo's nor a second plane's loads at 80 registers a
+// thread, and load latency (long scoreboard 3.7 of 9.5 cycles per instruction)
+// held the march at 55 % issue; taller stacks spilled (four lines: 256^3 513
+// -> 405 us, 192^3 283 -> 179, 144^3 143 -> 102).  The persistent batch keeps
+// registers (k_batch.cu).
 template <int NS, bool SMEM>
 struct RawSlots {
   double* own;  // slot i at own[i * blockDim.x]
@@ -83,7 +84,6 @@ struct RawSlots {
 // Slots: u*, w*, S of S lines, v* of S + 1 faces, (p^n, p^{n-1}, rho) of S lines
 // and of hn halo cells.
 __host__ __device__ constexpr int rhs_slots(int S, int hn) { return 3 * S + (S + 1) + 3 * S + 3 * hn; }
-__host__ __device__ constexpr bool rhs_slots_in_smem(int S) { return S <= 2; }
 
 // Column-stack form of the march for nx <= 512 (the same face and cell
 // arithmetic as k_rhs_march, bit for bit).  The CTA's threads form nstk =
@@ -399,7 +399,7 @@ __device__ __forceinline__ void rhs_stack_body(const GridDev& g, const StencilIn
 // 375 with either).  A third body in the same kernel, interior with the general
 // difference, brings that to 319 but costs the usual case registers: 384 x 256 x
 // 128 243 -> 256 us, 144^3 93 -> 97, and 128^3 with a caller's rho_0 55 -> 58.
-template <int S, int RULE, bool PROJ, int NXC = 0, bool SM = rhs_slots_in_smem(S)>
+template <int S, int RULE, bool PROJ, int NXC = 0, bool SM = true>
 __device__ __forceinline__ void rhs_stack_tile(const GridDev& g, const StencilIn& in, DevScalars* sc,
                                                const RhsOut& out, int kc, uint32_t bid) {
   const int tj = ((int)blockDim.x / (NXC ? NXC : g.nx)) * S;
